@@ -923,11 +923,10 @@ int adorym_l1_weights(adorym_ctx* ctx, int obj_id, double eps, float* w_delta, f
   if (ptr_kind(w_delta) != 1 || ptr_kind(w_beta) != 1) return fail(ctx, ADORYM_EINVAL, "weights must be device memory");
   const Object& o = it->second;
   const size_t n = (size_t)o.Lz * o.Ly * o.Lx;
-  int rc = ensure_ws(ctx, al(reg_parts(n) * sizeof(float)));
+  int rc = ensure_ws(ctx, al(2 * reg_parts(n) * sizeof(float)));
   if (rc) return rc;
   float* part = reinterpret_cast<float*>(ctx->ws);
-  cudaError_t e = launch_l1_weights(o.d, n, (float)eps, part, w_delta, ctx->stream);
-  if (e == cudaSuccess) e = launch_l1_weights(o.b, n, (float)eps, part, w_beta, ctx->stream);
+  const cudaError_t e = launch_l1_weights(o.d, o.b, n, (float)eps, part, w_delta, w_beta, ctx->stream);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "l1 weights");
   return ADORYM_OK;
 }

@@ -15,158 +15,148 @@ namespace adorym {
 
 __device__ __forceinline__ float sgn(float v) { return (v > 0.f) - (v < 0.f); }
 
-// One CTA per volume row (z, y) at a time (grid-stride over rows), threads along x: coalesced
-// loads, row and plane neighbours from L1/L2, and no per-voxel 64-bit index division.
-template <bool TV>
-__global__ void __launch_bounds__(256) k_regularize(const float* __restrict__ d, const float* __restrict__ b,
+// V consecutive floats of a row (V = 4: one 128-bit access, p 16-byte aligned)
+template <int V>
+__device__ __forceinline__ void load_v(float (&o)[V], const float* __restrict__ p) {
+  if constexpr (V == 4) {
+    const float4 v = *reinterpret_cast<const float4*>(p);
+    o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w;
+  } else {
+    o[0] = *p;
+  }
+}
+template <int V>
+__device__ __forceinline__ void store_v(float* __restrict__ p, const float (&o)[V]) {
+  if constexpr (V == 4) *reinterpret_cast<float4*>(p) = make_float4(o[0], o[1], o[2], o[3]);
+  else *p = o[0];
+}
+
+// Value and gradient.  A CTA takes a tile of 32 V x 8 columns (x, y) and walks zc planes of it: a warp
+// is one row, a thread V consecutive voxels.  The planes z - 1, z, z + 1 of delta and beta stay in
+// registers, the x neighbours come from the lanes beside (the tile's ends from one load), the y
+// neighbours from L1 where the tile holds them: 10 loads a voxel group instead of 14 + 4, and a fifth of
+// the L2 reads of a flat walk over the rows (which moved 60 bytes a voxel from L2 and was bound by it).
+// 512 x 512 x 32, weights, value and gradient (l1_weights and regularize): 192 -> 136 us; 80 registers
+// (three CTAs per SM), at 106 (two) 148 us.
+// V = 4 when Lx % 4 == 0 and the arrays are 16-byte aligned, else V = 1; the per-voxel arithmetic and
+// its order are the same.
+#ifndef REGB
+#define REGB 3
+#endif
+template <int V, bool TV>
+__global__ void __launch_bounds__(256, REGB) k_regularize(const float* __restrict__ d, const float* __restrict__ b,
                                                     const float* __restrict__ wd, const float* __restrict__ wb,
                                                     int Lz, int Ly, int Lx, float ad, float ab, float gam,
                                                     float invNo, float* __restrict__ gd, float* __restrict__ gb,
-                                                    double* __restrict__ part) {
+                                                    double* __restrict__ part, int zc) {
   __shared__ double red[8];
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const size_t sy = Lx, sz = (size_t)Lx * Ly;
-  const int rows = Ly * Lz;
+  const int gx = (Lx + 32 * V - 1) / (32 * V), gy = (Ly + 7) / 8, gz = (Lz + zc - 1) / zc;
+  const long long items = (long long)gx * gy * gz;
   Kahan acc;
-  for (int r = blockIdx.x; r < rows; r += gridDim.x) {
-    const int z = r / Ly, y = r - z * Ly;
-    const size_t base = (size_t)r * Lx;
-    for (int x = threadIdx.x; x < Lx; x += blockDim.x) {
-      const size_t i = base + x;
-      const float vd = d[i], vb = b[i];
-      const float w1 = wd ? wd[i] : 1.f, w2 = wb ? wb[i] : 1.f;
-      float term = ad * w1 * fabsf(vd) + ab * w2 * fabsf(vb);
-      float g1 = ad * w1 * sgn(vd), g2 = ab * w2 * sgn(vb);
+  for (long long item = blockIdx.x; item < items; item += gridDim.x) {
+    const int ix = (int)(item % gx), iy = (int)((item / gx) % gy), iz = (int)(item / ((long long)gx * gy));
+    const int x0 = (ix * 32 + lane) * V, y = iy * 8 + ty, z0 = iz * zc, z1 = min(z0 + zc, Lz);
+    const bool in = x0 < Lx && y < Ly;
+    size_t i = in ? ((size_t)z0 * Ly + y) * Lx + x0 : 0;
+    float cd[V] = {}, cb[V] = {}, pd[V] = {}, pb[V] = {}, nd[V] = {}, nb[V] = {};
+    if (in) {
+      load_v<V>(cd, d + i);
+      load_v<V>(cb, b + i);
+      if (TV && z0 > 0) {
+        load_v<V>(pd, d + i - sz);
+        load_v<V>(pb, b + i - sz);
+      }
+    }
+    for (int z = z0; z < z1; ++z, i += sz) {
+      float w1[V], w2[V], od[V] = {}, ob[V] = {}, ud[V] = {}, ub[V] = {}, vd[V] = {}, vb[V] = {};
+      float ld = 0.f, lb = 0.f, rd = 0.f, rb = 0.f;   // x neighbours beyond the warp's row piece
+#pragma unroll
+      for (int e = 0; e < V; ++e) w1[e] = w2[e] = 1.f;
+      if (in) {
+        if (z + 1 < (TV ? Lz : z1)) {
+          load_v<V>(nd, d + i + sz);
+          load_v<V>(nb, b + i + sz);
+        }
+        if (TV) {
+          if (y + 1 < Ly) {
+            load_v<V>(ud, d + i + sy);
+            load_v<V>(ub, b + i + sy);
+          }
+          if (y > 0) {
+            load_v<V>(vd, d + i - sy);
+            load_v<V>(vb, b + i - sy);
+          }
+          if (lane == 0 && x0 > 0) {
+            ld = d[i - 1];
+            lb = b[i - 1];
+          }
+          if (lane == 31 && x0 + V < Lx) {
+            rd = d[i + V];
+            rb = b[i + V];
+          }
+        }
+        if (wd) load_v<V>(w1, wd + i);
+        if (wb) load_v<V>(w2, wb + i);
+        if (gd) {
+          load_v<V>(od, gd + i);
+          load_v<V>(ob, gb + i);
+        }
+      }
       if (TV) {
-        const int pos[3] = {x, y, z}, lim[3] = {Lx, Ly, Lz};
-        const size_t st[3] = {1, sy, sz};
+        const float a = __shfl_up_sync(full, cd[V - 1], 1), c = __shfl_up_sync(full, cb[V - 1], 1);
+        const float f = __shfl_down_sync(full, cd[0], 1), g = __shfl_down_sync(full, cb[0], 1);
+        if (lane > 0) {
+          ld = a;
+          lb = c;
+        }
+        if (lane < 31) {
+          rd = f;
+          rb = g;
+        }
+      }
+      if (in) {
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-          if (pos[a] + 1 < lim[a]) {
-            const float fd = d[i + st[a]] - vd, fb = b[i + st[a]] - vb;
-            term += gam * (fabsf(fd) + fabsf(fb));
-            g1 -= gam * sgn(fd);
-            g2 -= gam * sgn(fb);
+        for (int e = 0; e < V; ++e) {
+          const float qd = cd[e], qb = cb[e];
+          float term = ad * w1[e] * fabsf(qd) + ab * w2[e] * fabsf(qb);
+          float g1 = ad * w1[e] * sgn(qd), g2 = ab * w2[e] * sgn(qb);
+          if (TV) {
+            auto ahead = [&](float hd, float hb) {   // forward difference of this voxel
+              const float fd = hd - qd, fb = hb - qb;
+              term += gam * (fabsf(fd) + fabsf(fb));
+              g1 -= gam * sgn(fd);
+              g2 -= gam * sgn(fb);
+            };
+            auto behind = [&](float hd, float hb) {   // forward difference of the voxel before
+              g1 += gam * sgn(qd - hd);
+              g2 += gam * sgn(qb - hb);
+            };
+            if (x0 + e + 1 < Lx) ahead(e + 1 < V ? cd[(e + 1) % V] : rd, e + 1 < V ? cb[(e + 1) % V] : rb);
+            if (x0 + e > 0) behind(e > 0 ? cd[(e + V - 1) % V] : ld, e > 0 ? cb[(e + V - 1) % V] : lb);
+            if (y + 1 < Ly) ahead(ud[e], ub[e]);
+            if (y > 0) behind(vd[e], vb[e]);
+            if (z + 1 < Lz) ahead(nd[e], nb[e]);
+            if (z > 0) behind(pd[e], pb[e]);
           }
-          if (pos[a] > 0) {
-            g1 += gam * sgn(vd - d[i - st[a]]);
-            g2 += gam * sgn(vb - b[i - st[a]]);
-          }
+          acc.add(term);
+          od[e] += g1 * invNo;
+          ob[e] += g2 * invNo;
+        }
+        if (gd) {
+          store_v<V>(gd + i, od);
+          store_v<V>(gb + i, ob);
         }
       }
-      acc.add(term);
-      if (gd) {
-        gd[i] += g1 * invNo;
-        gb[i] += g2 * invNo;
+#pragma unroll
+      for (int e = 0; e < V; ++e) {
+        pd[e] = cd[e];
+        pb[e] = cb[e];
+        cd[e] = nd[e];
+        cb[e] = nb[e];
       }
-    }
-  }
-  double v = acc.value();
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int k = 0; k < 8; ++k) s += red[k];
-    part[blockIdx.x] = s;
-  }
-}
-
-// The same value and gradient with four consecutive voxels of a row per thread (Lx % 4 == 0 and
-// 16-byte aligned arrays): 128-bit loads of delta, beta, the weights, the neighbour rows and
-// planes and the gradients, the x neighbours across the group from two scalar loads.  Same
-// per-voxel arithmetic and the same Kahan order within a thread as k_regularize.
-template <bool TV>
-__global__ void __launch_bounds__(256) k_regularize4(const float* __restrict__ d, const float* __restrict__ b,
-                                                     const float* __restrict__ wd, const float* __restrict__ wb,
-                                                     int Lz, int Ly, int Lx, float ad, float ab, float gam,
-                                                     float invNo, float* __restrict__ gd, float* __restrict__ gb,
-                                                     double* __restrict__ part) {
-  __shared__ double red[8];
-  const int Lx4 = Lx >> 2;
-  const size_t sy = Lx, sz = (size_t)Lx * Ly;
-  const size_t n4 = (size_t)Ly * Lz * Lx4;
-  const float4 one4 = make_float4(1.f, 1.f, 1.f, 1.f);
-  Kahan acc;
-  for (size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x; q < n4; q += (size_t)gridDim.x * blockDim.x) {
-    const int r = (int)(q / Lx4), x0 = 4 * (int)(q - (size_t)r * Lx4);
-    const int z = r / Ly, y = r - z * Ly;
-    const size_t i = (size_t)r * Lx + x0;
-    const float4 vd = *reinterpret_cast<const float4*>(d + i), vb = *reinterpret_cast<const float4*>(b + i);
-    const float4 w1 = wd ? *reinterpret_cast<const float4*>(wd + i) : one4;
-    const float4 w2 = wb ? *reinterpret_cast<const float4*>(wb + i) : one4;
-    const float cd[4] = {vd.x, vd.y, vd.z, vd.w}, cb[4] = {vb.x, vb.y, vb.z, vb.w};
-    const float cw1[4] = {w1.x, w1.y, w1.z, w1.w}, cw2[4] = {w2.x, w2.y, w2.z, w2.w};
-    float term[4], g1[4], g2[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      term[e] = ad * cw1[e] * fabsf(cd[e]) + ab * cw2[e] * fabsf(cb[e]);
-      g1[e] = ad * cw1[e] * sgn(cd[e]);
-      g2[e] = ab * cw2[e] * sgn(cb[e]);
-    }
-    if (TV) {
-      // x neighbours: within the group, and one scalar on each side
-      float nd[6], nb[6];   // nd[e + 1] = delta at x0 + e, e = -1..4
-      nd[0] = x0 > 0 ? d[i - 1] : 0.f;
-      nb[0] = x0 > 0 ? b[i - 1] : 0.f;
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        nd[e + 1] = cd[e];
-        nb[e + 1] = cb[e];
-      }
-      nd[5] = x0 + 4 < Lx ? d[i + 4] : 0.f;
-      nb[5] = x0 + 4 < Lx ? b[i + 4] : 0.f;
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int x = x0 + e;
-        if (x + 1 < Lx) {
-          const float fd = nd[e + 2] - cd[e], fb = nb[e + 2] - cb[e];
-          term[e] += gam * (fabsf(fd) + fabsf(fb));
-          g1[e] -= gam * sgn(fd);
-          g2[e] -= gam * sgn(fb);
-        }
-        if (x > 0) {
-          g1[e] += gam * sgn(cd[e] - nd[e]);
-          g2[e] += gam * sgn(cb[e] - nb[e]);
-        }
-      }
-      // y and z neighbours: whole groups of the adjacent rows and planes
-      const int pos[2] = {y, z}, lim[2] = {Ly, Lz};
-      const size_t st[2] = {sy, sz};
-#pragma unroll
-      for (int a = 0; a < 2; ++a) {
-        if (pos[a] + 1 < lim[a]) {
-          const float4 ud = *reinterpret_cast<const float4*>(d + i + st[a]);
-          const float4 ub = *reinterpret_cast<const float4*>(b + i + st[a]);
-          const float qd[4] = {ud.x, ud.y, ud.z, ud.w}, qb[4] = {ub.x, ub.y, ub.z, ub.w};
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const float fd = qd[e] - cd[e], fb = qb[e] - cb[e];
-            term[e] += gam * (fabsf(fd) + fabsf(fb));
-            g1[e] -= gam * sgn(fd);
-            g2[e] -= gam * sgn(fb);
-          }
-        }
-        if (pos[a] > 0) {
-          const float4 ud = *reinterpret_cast<const float4*>(d + i - st[a]);
-          const float4 ub = *reinterpret_cast<const float4*>(b + i - st[a]);
-          const float qd[4] = {ud.x, ud.y, ud.z, ud.w}, qb[4] = {ub.x, ub.y, ub.z, ub.w};
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            g1[e] += gam * sgn(cd[e] - qd[e]);
-            g2[e] += gam * sgn(cb[e] - qb[e]);
-          }
-        }
-      }
-    }
-#pragma unroll
-    for (int e = 0; e < 4; ++e) acc.add(term[e]);
-    if (gd) {
-      float4 od = *reinterpret_cast<float4*>(gd + i), ob = *reinterpret_cast<float4*>(gb + i);
-      od.x += g1[0] * invNo; od.y += g1[1] * invNo; od.z += g1[2] * invNo; od.w += g1[3] * invNo;
-      ob.x += g2[0] * invNo; ob.y += g2[1] * invNo; ob.z += g2[2] * invNo; ob.w += g2[3] * invNo;
-      *reinterpret_cast<float4*>(gd + i) = od;
-      *reinterpret_cast<float4*>(gb + i) = ob;
     }
   }
   double v = acc.value();
@@ -199,77 +189,121 @@ __global__ void __launch_bounds__(256) k_reg_final(const double* __restrict__ pa
   }
 }
 
-// max |C| over the volume: per-CTA maxima, then one CTA (|C| >= 0, so float order = bit order)
-__global__ void __launch_bounds__(256) k_absmax(const float* __restrict__ c, size_t n, float* __restrict__ part) {
+// max |C| of delta (blockIdx.y = 0) and beta (1): per-CTA maxima (NaNs are passed over, as by fmaxf)
+template <int V>
+__global__ void __launch_bounds__(256) k_absmax(const float* __restrict__ cd, const float* __restrict__ cb, size_t n,
+                                                float* __restrict__ part) {
   __shared__ float red[8];
+  const float* __restrict__ c = blockIdx.y ? cb : cd;
+  constexpr int U = 4;   // loads in flight per thread
+  const size_t nv = n / V, step = (size_t)gridDim.x * blockDim.x;
   float m = 0.f;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-    m = fmaxf(m, fabsf(c[i]));
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nv; i += U * step) {
+    float v[U][V];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+#pragma unroll
+      for (int e = 0; e < V; ++e) v[u][e] = 0.f;
+      if (i + u * step < nv) load_v<V>(v[u], c + (i + u * step) * V);
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int e = 0; e < V; ++e) m = fmaxf(m, fabsf(v[u][e]));
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int k = 1; k < 8; ++k) m = fmaxf(m, red[k]);
-    part[blockIdx.x] = m;
+    part[blockIdx.y * gridDim.x + blockIdx.x] = m;
   }
 }
 
-__global__ void __launch_bounds__(256) k_l1_weights(const float* __restrict__ c, size_t n,
+// W = max|C| / (|C| + eps) of both volumes.  Every CTA takes the maximum of the nparts partials with
+// all of its threads: walked by one thread it was 30 of the 37 us of a 512 x 512 x 32 volume.
+template <int V>
+__global__ void __launch_bounds__(256) k_l1_weights(const float* __restrict__ cd, const float* __restrict__ cb, size_t n,
                                                     const float* __restrict__ part, int nparts, float eps,
-                                                    float* __restrict__ w) {
-  __shared__ float mx;
-  if (threadIdx.x == 0) {
-    float m = 0.f;
-    for (int k = 0; k < nparts; ++k) m = fmaxf(m, part[k]);
-    mx = m;
-  }
+                                                    float* __restrict__ wd, float* __restrict__ wb) {
+  __shared__ float red[8];
+  const float* __restrict__ c = blockIdx.y ? cb : cd;
+  float* __restrict__ w = blockIdx.y ? wb : wd;
+  float m = 0.f;
+  for (int k = threadIdx.x; k < nparts; k += 256) m = fmaxf(m, part[blockIdx.y * nparts + k]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
   __syncthreads();
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-    w[i] = mx / (fabsf(c[i]) + eps);
+  float mx = red[0];
+#pragma unroll
+  for (int k = 1; k < 8; ++k) mx = fmaxf(mx, red[k]);
+  constexpr int U = 4;
+  const size_t nv = n / V, step = (size_t)gridDim.x * blockDim.x;
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nv; i += U * step) {
+    float v[U][V];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (i + u * step < nv) load_v<V>(v[u], c + (i + u * step) * V);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (i + u * step >= nv) break;
+#pragma unroll
+      for (int e = 0; e < V; ++e) v[u][e] = mx / (fabsf(v[u][e]) + eps);
+      store_v<V>(w + (i + u * step) * V, v[u]);
+    }
+  }
 }
 
 static unsigned reg_grid(size_t n) { return (unsigned)std::min<size_t>((n + 255) / 256, 152 * 8); }
 
 int reg_parts(size_t n) { return (int)reg_grid(n); }
 
-// rows of the regularizer kernel: at most reg_grid(n) CTAs (its partial-sum array), one row each
-static unsigned reg_rows_grid(int Ly, int Lz, size_t n) {
-  return (unsigned)std::min<size_t>((size_t)Ly * Lz, reg_grid(n));
-}
+static bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
 cudaError_t launch_regularize(const float* d, const float* b, const float* wd, const float* wb, int Lz, int Ly, int Lx,
                               double ad, double ab, double gam, float* gd, float* gb, double* part, double* loss,
                               cudaStream_t s) {
   const size_t n = (size_t)Lz * Ly * Lx;
   const float invNo = (float)(1.0 / (double)n);
-  auto al16 = [](const void* p) { return ((uintptr_t)p & 15u) == 0; };
-  if (Lx % 4 == 0 && al16(d) && al16(b) && (!wd || al16(wd)) && (!wb || al16(wb)) && (!gd || (al16(gd) && al16(gb)))) {
-    const unsigned grid = reg_grid(n);
-    if (gam != 0.0)
-      (k_regularize4<true><<<grid, 256, 0, s>>>(d, b, wd, wb, Lz, Ly, Lx, (float)ad, (float)ab, (float)gam, invNo, gd,
-                                                gb, part), note_launch());
-    else
-      (k_regularize4<false><<<grid, 256, 0, s>>>(d, b, wd, wb, Lz, Ly, Lx, (float)ad, (float)ab, 0.f, invNo, gd, gb,
-                                                 part), note_launch());
-    if (loss) (k_reg_final<<<1, 256, 0, s>>>(part, (int)grid, 1.0 / (double)n, loss), note_launch());
-    return cudaGetLastError();
-  }
-  const unsigned grid = reg_rows_grid(Ly, Lz, n);
-  if (gam != 0.0)
-    (k_regularize<true><<<grid, 256, 0, s>>>(d, b, wd, wb, Lz, Ly, Lx, (float)ad, (float)ab, (float)gam, invNo, gd,
-                                             gb, part), note_launch());
-  else
-    (k_regularize<false><<<grid, 256, 0, s>>>(d, b, wd, wb, Lz, Ly, Lx, (float)ad, (float)ab, 0.f, invNo, gd, gb,
-                                              part), note_launch());
+  const bool vec = Lx % 4 == 0 && aligned16(d) && aligned16(b) && aligned16(wd) && aligned16(wb) && aligned16(gd) && aligned16(gb);
+  const int V = vec ? 4 : 1;
+  // planes per tile: as many as leave the chip eight CTAs per SM (fewer planes re-read more of their neighbours)
+  const long long tiles = (long long)((Lx + 32 * V - 1) / (32 * V)) * ((Ly + 7) / 8);
+  int zc = 16;
+  while (zc > 2 && tiles * ((Lz + zc - 1) / zc) < 152 * 8) zc /= 2;
+  const unsigned grid = (unsigned)std::min<long long>(tiles * ((Lz + zc - 1) / zc), reg_grid(n));
+  auto run = [&](auto kernel, float g) {
+    (kernel<<<grid, 256, 0, s>>>(d, b, wd, wb, Lz, Ly, Lx, (float)ad, (float)ab, g, invNo, gd, gb, part, zc), note_launch());
+  };
+  if (gam != 0.0) vec ? run(k_regularize<4, true>, (float)gam) : run(k_regularize<1, true>, (float)gam);
+  else vec ? run(k_regularize<4, false>, 0.f) : run(k_regularize<1, false>, 0.f);
   if (loss) (k_reg_final<<<1, 256, 0, s>>>(part, (int)grid, 1.0 / (double)n, loss), note_launch());
   return cudaGetLastError();
 }
 
-cudaError_t launch_l1_weights(const float* c, size_t n, float eps, float* part, float* w, cudaStream_t s) {
-  const unsigned grid = reg_grid(n);
-  (k_absmax<<<grid, 256, 0, s>>>(c, n, part), note_launch());
-  (k_l1_weights<<<grid, 256, 0, s>>>(c, n, part, (int)grid, eps, w), note_launch());
+cudaError_t launch_l1_weights(const float* d, const float* b, size_t n, float eps, float* part, float* wd, float* wb,
+                              cudaStream_t s) {
+  const bool vec = n % 4 == 0 && aligned16(d) && aligned16(b) && aligned16(wd) && aligned16(wb);
+  const unsigned grid = std::min(reg_grid(n), 152u * 4);   // per volume
+  auto run = [&](unsigned volumes, const float* c0, float* w0) {
+    const dim3 g(grid, volumes);
+    if (vec) {
+      (k_absmax<4><<<g, 256, 0, s>>>(c0, b, n, part), note_launch());
+      (k_l1_weights<4><<<g, 256, 0, s>>>(c0, b, n, part, (int)grid, eps, w0, wb), note_launch());
+    } else {
+      (k_absmax<1><<<g, 256, 0, s>>>(c0, b, n, part), note_launch());
+      (k_l1_weights<1><<<g, 256, 0, s>>>(c0, b, n, part, (int)grid, eps, w0, wb), note_launch());
+    }
+  };
+  auto overlap = [n](const float* p, const float* q) { return p < q + n && q < p + n; };
+  if (overlap(wd, wb) || overlap(wd, b) || overlap(wb, d)) {   // one volume after the other (one buffer for both, say)
+    run(1, d, wd);
+    run(1, b, wb);
+  } else {
+    run(2, d, wd);
+  }
   return cudaGetLastError();
 }
 

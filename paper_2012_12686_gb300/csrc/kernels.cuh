@@ -200,8 +200,9 @@ int reg_parts(size_t n);
 cudaError_t launch_regularize(const float* d, const float* b, const float* wd, const float* wb, int Lz, int Ly, int Lx,
                               double ad, double ab, double gam, float* gd, float* gb, double* part, double* loss,
                               cudaStream_t s);
-// W = max|C| / (|C| + eps); part needs reg_parts(n) floats
-cudaError_t launch_l1_weights(const float* c, size_t n, float eps, float* part, float* w, cudaStream_t s);
+// W = max|C| / (|C| + eps) for C = delta and beta; part needs 2 reg_parts(n) floats
+cudaError_t launch_l1_weights(const float* d, const float* b, size_t n, float eps, float* part, float* wd, float* wb,
+                              cudaStream_t s);
 // qsum[i] = sum_b qacc[b][i] in FP64, fixed order
 cudaError_t launch_qsum(const float2* qacc, float2* qsum, int B, size_t MNN, cudaStream_t s);
 int path_smem_bytes(int N);
