@@ -25,9 +25,7 @@
 // After C2, smem row r holds y-frequency  r / N2 + N1 * (r % N2).
 //
 // Twiddles W_N^m = exp(-2 pi i m / N) come from a table built in FP64 on the
-// host and rounded once to FP32 (at N = 128 rearranged per stage so that a task
-// reads two of them per 128-bit shared load); the in-register DFT_R (R <= 16)
-// uses compile-time constants of exp(+-2 pi i k / 16).
+// host and rounded once to FP32; the in-register DFT_R uses compile-time constants of exp(+-2 pi i k / 16).
 #pragma once
 #include <cuda_runtime.h>
 #include <utility>
@@ -162,45 +160,15 @@ struct Geo;
 // NT threads per CTA; MINB resident CTAs per SM the register budget is sized for (128 regs/thread)
 // The spatial passes (S4/S1, radix N1) carry the global-memory traffic of the pointwise ops, so
 // N1 is the smaller radix where the two differ.
-#ifndef ADORYM_NT128
-#define ADORYM_NT128 512
-#endif
-// ADORYM_FOURPASS64: N = 64 fused kernels on the four-pass scheme of fft_block4.cuh (256 threads).
-// Off by default: its radix-16 stages raised the full-size tomography probe-gradient error above
-// the stored FP32 floor (1.68e-3 against a bar of 1.58e-3; the radix-8 stages of the default form
-// give 1.49e-3), and the one tomography launch measured with it (scalar arithmetic) took 1.35 ms
-// against 1.22 ms for the packed six-pass form of the time.
-#ifndef ADORYM_FOURPASS64
-#define ADORYM_FOURPASS64 0
-#endif
-#ifndef ADORYM_NT64
-#define ADORYM_NT64 (ADORYM_FOURPASS64 ? 256 : 512)
-#endif
 template <> struct Geo<8>   { static constexpr int N1 = 4, N2 = 2,  NT = 64,  MINB = 8; };
 template <> struct Geo<16>  { static constexpr int N1 = 4, N2 = 4,  NT = 64,  MINB = 8; };
 template <> struct Geo<32>  { static constexpr int N1 = 4, N2 = 8,  NT = 128, MINB = 4; };
-template <> struct Geo<64>  { static constexpr int N1 = 8, N2 = 8,  NT = ADORYM_NT64, MINB = 512 / ADORYM_NT64; };
-template <> struct Geo<128> { static constexpr int N1 = 8, N2 = 16, NT = ADORYM_NT128, MINB = 1; };
+template <> struct Geo<64>  { static constexpr int N1 = 8, N2 = 8,  NT = 512, MINB = 1; };
+template <> struct Geo<128> { static constexpr int N1 = 8, N2 = 16, NT = 512, MINB = 1; };
 
 template <int N>
 struct Field {
   static constexpr int N1 = Geo<N>::N1, N2 = Geo<N>::N2, NT = Geo<N>::NT, LD = N + 1;
-  static constexpr int SMEM_FLOAT2 = N * LD;
-  // shared twiddle tables at tw (16-byte aligned): tw[m] = W_N^m (m < N); at N = 128 also the
-  // S1/S4-side table [N2][N1] at tw + N and the S3-side table [N1][N2] at tw + 2N (entries
-  // W_N^(t k)), which the passes read two twiddles per access (fewer shared-memory instructions,
-  // -2 % time); at N = 64 the single-twiddle reads of tw measured faster
-  static constexpr bool PAIRED_TW = N >= 128;
-  static constexpr int TW_ENTRIES = PAIRED_TW ? 3 * N : N;
-  __device__ static __forceinline__ void fill_twiddles(float2* tw, const float2* __restrict__ twg) {
-    for (int i = threadIdx.x; i < N; i += NT) {
-      tw[i] = twg[i];
-      if (PAIRED_TW) {
-        tw[N + i] = twg[(i / N1) * (i % N1)];
-        tw[2 * N + i] = twg[(i / N2) * (i % N2)];
-      }
-    }
-  }
   // y-frequency held by smem row r after the column forward stages (C2)
   __device__ static __forceinline__ int row_freq(int r) { return r / N2 + N1 * (r % N2); }
 };
@@ -209,7 +177,7 @@ struct Field {
 // Passes.  Signs are compile-time: S = -1 (DFT_-), +1 (DFT_+), 0 (stage skipped).
 //
 // Column pass "14": tasks (x, t < N2); v[k] <-> sample y = N2*k + t.
-//   pre(pa, pb, x, t): issues the task's global loads before the smem loads and S4
+//   pre(pa, pb, x, t): issues the task's global loads, before the CTA barrier that opens the pass
 //   op(v, pa, pb, x, t): spatial pointwise op on natural samples
 //   S1 != 0: S1 then store; S1 == 0: store natural samples; STORE = false: no store
 // LOAD = false: the samples come from op (no smem read, no S4).
@@ -234,17 +202,22 @@ __device__ __forceinline__ void pass_c14(float2* __restrict__ A, const float2* _
   using F = Field<N>;
   constexpr int N1 = F::N1, N2 = F::N2, LD = F::LD;
   using P = Tpt<N * N2, F::NT>;
-  // the spatial pass keeps three register arrays per task; phase its tasks only when they fit
-  constexpr int Q = (F::NT <= 512) ? (P::n < 2 ? P::n : 2) : 1;
+  // the spatial pass keeps three register arrays per task: at most two tasks at a time
+  constexpr int Q = P::n < 2 ? P::n : 2;
   for (int q0 = 0; q0 < P::n; q0 += Q) {
     float2 pa[Q][N1], pb[Q][N1], v[Q][N1];
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
       const int tau = threadIdx.x + (q0 + q) * F::NT;
-      if (!P::ok(tau)) continue;
-      const int x = tau % N, t = tau / N;
-      pre(pa[q], pb[q], x, t);
-      if (LOAD) {
+      if (P::ok(tau)) pre(pa[q], pb[q], tau % N, tau / N);
+    }
+    if (q0 == 0) __syncthreads();
+    if (LOAD) {
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        const int tau = threadIdx.x + (q0 + q) * F::NT;
+        if (!P::ok(tau)) continue;
+        const int x = tau % N, t = tau / N;
 #pragma unroll
         for (int i = 0; i < N1; ++i) v[q][i] = A[(N2 * i + t) * LD + x];
       }
@@ -258,8 +231,7 @@ __device__ __forceinline__ void pass_c14(float2* __restrict__ A, const float2* _
       op(v[q], pa[q], pb[q], x, t);
       if (STORE && S1) {
         dft<N1, S1>(v[q]);
-        if constexpr (F::PAIRED_TW) twiddle_row<S1, N1>(v[q], tw + N + t * N1);
-        else twiddle<S1>(v[q], tw, t);
+        twiddle<S1>(v[q], tw, t);
       }
     }
     if (STORE) {
@@ -297,8 +269,7 @@ __device__ __noinline__ void pass_c23(float2* __restrict__ A, const float2* __re
     const int t = tau / N;
     dft<N2, S>(v[q]);
     if constexpr (IS_S3) {
-      if constexpr (F::PAIRED_TW) twiddle_row<S, N2>(v[q], tw + 2 * N + t * N2);
-      else twiddle<S>(v[q], tw, t);
+      twiddle<S>(v[q], tw, t);
     }
   }
 #pragma unroll
@@ -333,8 +304,7 @@ __device__ __noinline__ void pass_r14(float2* __restrict__ A, const float2* __re
     const int t = tau / N;
     dft<N1, S>(v[q]);
     if constexpr (IS_S1) {
-      if constexpr (F::PAIRED_TW) twiddle_row<S, N1>(v[q], tw + N + t * N1);
-      else twiddle<S>(v[q], tw, t);
+      twiddle<S>(v[q], tw, t);
     }
   }
 #pragma unroll
@@ -376,8 +346,7 @@ __device__ __forceinline__ void pass_r23(float2* __restrict__ A, const float2* _
     op(v[q], F::row_freq(r), t);
     if (S3) {
       dft<N2, S3>(v[q]);
-      if constexpr (F::PAIRED_TW) twiddle_row<S3, N2>(v[q], tw + 2 * N + t * N2);
-      else twiddle<S3>(v[q], tw, t);
+      twiddle<S3>(v[q], tw, t);
     }
   }
   if (S3) {

@@ -1,36 +1,45 @@
 // Launchers of the fused kernel without per-gap propagators, and the per-call probe kernels
 // around it (probe DFT, probe-gradient reduction, slice-gap gradient reduction).
+#include <algorithm>
+#include <type_traits>
+
 #include "k_path.cuh"
 
 namespace adorym {
 
 // ---------------------------------------------------------------------------- probe DFT
+// The probe's spectrum enters every transform that follows, so its stages stay 8 x 16 at N = 128: the
+// four-pass radices round differently, and the object and probe gradients of a 32-slice batch moved by
+// 6e-6 of their norm.
+template <int N>
+using ProbeFFT = std::conditional_t<N == 128, SixPass<N>, PathFFT<N>>;
+
 template <int N>
 __global__ void __launch_bounds__(Geo<N>::NT) k_probe_hat(const float2* __restrict__ probe, float2* __restrict__ phat,
                                                         const float2* __restrict__ twg) {
-  using F = Field<N>;
-  constexpr int N1 = F::N1, N2 = F::N2;
+  using X = ProbeFFT<N>;
+  constexpr int CY = X::CY, YS = X::YS, RX = X::RX, KXS = X::KXS;
   extern __shared__ float2 sm[];
   float2* A = sm;
-  float2* tw = A + N * F::LD;
-  F::fill_twiddles(tw, twg);
-  __syncthreads();
+  float2* tw = A + X::FIELD;
+  X::fill_twiddles(tw, twg);
   const float2* p = probe + (size_t)blockIdx.x * N * N;
   float2* o = phat + (size_t)blockIdx.x * N * N;
-  using V1 = float2[N1];
-  using V2 = float2[N2];
-  pass_c14<N, 0, -1, false, true>(A, tw, NoPre(), [&](V1& v, V1&, V1&, int x, int t) {
+  using V1 = float2[CY];
+  using V2 = float2[RX];
+  X::template c14<0, -1, false, true>(A, tw, [&](V1&, V1& pb, int x, int t) {
 #pragma unroll
-    for (int k = 0; k < N1; ++k) v[k] = p[(N2 * k + t) * N + x];
+    for (int k = 0; k < CY; ++k) pb[k] = __ldg(p + (YS * k + t) * N + x);
+  }, [&](V1& v, V1&, V1& pb, int, int) {
+#pragma unroll
+    for (int k = 0; k < CY; ++k) v[k] = pb[k];
   });
   __syncthreads();
-  pass_c23<N, false, -1>(A, tw);
-  __syncthreads();
-  pass_r14<N, true, -1>(A, tw);
-  __syncthreads();
-  pass_r23<N, -1, 0>(A, tw, [&](V2& v, int ky, int t) {
+  X::template fwd_pair<-1>(A, tw);
+  X::row_sync();
+  X::template r23<-1, 0>(A, tw, [&](V2& v, int ky, int t) {
 #pragma unroll
-    for (int i = 0; i < N2; ++i) o[ky * N + t + N1 * i] = v[i];
+    for (int i = 0; i < RX; ++i) o[ky * N + t + KXS * i] = v[i];
   });
 }
 
@@ -116,12 +125,12 @@ template <int N, int FAR>
 __global__ void __launch_bounds__(Geo<N>::NT) k_probe_grad(const float2* __restrict__ qsum, float2* __restrict__ g,
                                                          const float2* __restrict__ twg, const double* __restrict__ lossp,
                                                          int B, double inv_npix, double* __restrict__ loss_out) {
-  using F = Field<N>;
-  constexpr int N1 = F::N1, N2 = F::N2, NT = F::NT;
+  using X = PathFFT<N>;
+  constexpr int CY = X::CY, YS = X::YS, RX = X::RX, KXS = X::KXS, NT = Geo<N>::NT;
   constexpr size_t NN = (size_t)N * N;
   extern __shared__ float2 sm[];
   float2* A = sm;
-  float2* tw = A + N * F::LD;
+  float2* tw = A + X::FIELD;
   if (loss_out && blockIdx.x == 0 && threadIdx.x < 32) {
     // FP64 sum of the per-position partials in a fixed order: lane l adds positions l, l + 32, ...
     // in turn, then a fixed xor tree over the lanes (one warp keeps B / 32 loads in flight instead of
@@ -139,26 +148,23 @@ __global__ void __launch_bounds__(Geo<N>::NT) k_probe_grad(const float2* __restr
     for (size_t i = threadIdx.x; i < NN; i += NT) o[i] = cadd(o[i], q[i]);
     return;
   }
-  F::fill_twiddles(tw, twg);
+  X::fill_twiddles(tw, twg);
   __syncthreads();
   const float invNN = 1.0f / (float)NN;
-  using V1 = float2[N1];
-  using V2 = float2[N2];
-  pass_r23<N, 0, +1>(A, tw, [&](V2& v, int ky, int t) {
+  using V1 = float2[CY];
+  using V2 = float2[RX];
+  X::template r23<0, +1>(A, tw, [&](V2& v, int ky, int t) {
 #pragma unroll
-    for (int i = 0; i < N2; ++i) v[i] = cscale(q[ky * N + t + N1 * i], invNN);
+    for (int i = 0; i < RX; ++i) v[i] = cscale(__ldg(q + ky * N + t + KXS * i), invNN);
   });
-  __syncthreads();
-  pass_r14<N, false, +1>(A, tw);
-  __syncthreads();
-  pass_c23<N, true, +1>(A, tw);
-  __syncthreads();
-  pass_c14<N, +1, 0, true, false>(A, tw, NoPre(), [&](V1& v, V1&, V1&, int x, int t) {
+  X::row_sync();
+  X::template inv_pair<+1>(A, tw);
+  X::template c14<+1, 0, true, false>(A, tw, [&](V1& pa, V1&, int x, int t) {
 #pragma unroll
-    for (int k = 0; k < N1; ++k) {
-      const int p = (N2 * k + t) * N + x;
-      o[p] = cadd(o[p], v[k]);
-    }
+    for (int k = 0; k < CY; ++k) pa[k] = o[(YS * k + t) * N + x];
+  }, [&](V1& v, V1& pa, V1&, int x, int t) {
+#pragma unroll
+    for (int k = 0; k < CY; ++k) o[(YS * k + t) * N + x] = cadd(pa[k], v[k]);
   });
 }
 
@@ -194,8 +200,13 @@ cudaError_t launch_path(const PathArgs& a, int farfield, cudaStream_t s) {
 }
 
 template <int N>
+constexpr int probe_smem_bytes() {   // field + twiddle tables
+  return std::max(PathFFT<N>::FIELD + PathFFT<N>::TW, ProbeFFT<N>::FIELD + ProbeFFT<N>::TW) * (int)sizeof(float2);
+}
+
+template <int N>
 static cudaError_t launch_probe_hat_t(int M, const float2* probe, float2* phat, const float2* tw, cudaStream_t s) {
-  const int smem = (N * (N + 1) + Field<N>::TW_ENTRIES) * (int)sizeof(float2);
+  const int smem = probe_smem_bytes<N>();
   (k_probe_hat<N><<<M, Geo<N>::NT, smem, s>>>(probe, phat, tw), note_launch());
   return cudaGetLastError();
 }
@@ -218,7 +229,7 @@ static cudaError_t launch_probe_grad_t(int M, int B, const float2* qacc, float2*
   if (g) {
     (k_qsum<<<(unsigned)((MNN + 31) / 32), 256, 0, s>>>(qacc, qsum, B, MNN), note_launch());
   }
-  const int smem = (N * (N + 1) + Field<N>::TW_ENTRIES) * (int)sizeof(float2);
+  const int smem = probe_smem_bytes<N>();
   (k_probe_grad<N, FAR><<<M, Geo<N>::NT, smem, s>>>(qsum, g, tw, lossp, B, inv_npix, loss_out), note_launch());
   return cudaGetLastError();
 }
@@ -248,7 +259,7 @@ static cudaError_t prepare_t() {
   if (e == cudaSuccess) e = prepare_path_gaps(N, FAR);
   if (e == cudaSuccess) e = prepare_path_pipe(N, FAR);
   if (e == cudaSuccess) e = prepare_path_help(N, FAR);
-  const int small = (N * (N + 1) + Field<N>::TW_ENTRIES) * (int)sizeof(float2);
+  const int small = probe_smem_bytes<N>();
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_probe_hat<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, small);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_probe_grad<N, FAR>, cudaFuncAttributeMaxDynamicSharedMemorySize, small);
   return e;

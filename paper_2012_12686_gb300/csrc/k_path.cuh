@@ -125,14 +125,14 @@ __device__ __forceinline__ void path_body(const PathArgs& a) {
   static_assert(!(HELP && (GAP || PIPE)), "recompute helpers serve the plain one-CTA form only");
   using F = Field<N>;
   using X = PathFFT<N>;
-  constexpr int CY = X::CY, YS = X::YS, RX = X::RX, KXS = X::KXS, LD = F::LD, NT = F::NT;
+  constexpr int CY = X::CY, YS = X::YS, RX = X::RX, KXS = X::KXS, NT = F::NT;
   constexpr size_t NN = (size_t)N * N;
   using V1 = float2[CY];
   using V2 = float2[RX];
   extern __shared__ float2 sm[];
   float2* A = sm;
-  float2* tw = A + N * LD;             // F::TW_ENTRIES twiddles (tw, then the per-stage tables)
-  float2* hy = tw + F::TW_ENTRIES;
+  float2* tw = A + X::FIELD;
+  float2* hy = tw + X::TW;
   float2* hx = hy + N;
   float2* ry = hx + N;
   float2* rx = ry + N;
@@ -142,7 +142,7 @@ __device__ __forceinline__ void path_body(const PathArgs& a) {
   const int b = PIPE ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
   const int rank = PIPE ? (int)(blockIdx.x & 1) : 0;   // cluster of two CTAs along x
   const int M = a.M, L = a.L, cp = a.cp, ncp = a.ncp;
-  F::fill_twiddles(tw, a.tw);
+  X::fill_twiddles(tw, a.tw);
   for (int i = threadIdx.x; i < N; i += NT) {
     hy[i] = a.hy[i];
     hx[i] = a.hx[i];
@@ -194,7 +194,7 @@ __device__ __forceinline__ void path_body(const PathArgs& a) {
   // accumulates dL/dc_gap = -pi sum |f|^2 Im(conj(F[psibar]) F[psi]) into gapp
   auto propagate_tail = [&](bool adjoint, int gapj, float2* spec_out, const float2* spec_in) {
     X::template fwd_pair<-1>(A, tw);
-    __syncthreads();
+    X::row_sync();
     float gs = 0.f;
     if constexpr (GAP) {
       const float2* hyp = a.hyj + (size_t)gapj * N;
@@ -231,9 +231,8 @@ __device__ __forceinline__ void path_body(const PathArgs& a) {
         for (int i = 0; i < RX; ++i) v[i] = cmul(cmul(v[i], h), hx[t + KXS * i]);
       });
     }
-    __syncthreads();
+    X::row_sync();
     X::template inv_pair<+1>(A, tw);
-    __syncthreads();
     if constexpr (GAP) {
       if (adjoint && spec_in) {
         const double g = block_sum<NT>(f32_to_f64(gs), red);
@@ -306,9 +305,8 @@ __device__ __forceinline__ void path_body(const PathArgs& a) {
           v[i] = cmul(cmul(__ldg(&ph[ky * N + kx]), r), rx[kx]);
         }
       });
-      __syncthreads();
+      X::row_sync();
       X::template inv_pair<+1>(A, tw);
-      __syncthreads();
     }
     for (int j = 0; j < L; ++j) {
       const bool last = (j == L - 1);
@@ -341,7 +339,7 @@ __device__ __forceinline__ void path_body(const PathArgs& a) {
       if (FAR) {
         // Psi = (1/N) DFT_+[phi]; keep Psi, accumulate I over modes
         X::template fwd_pair<+1>(A, tw);
-        __syncthreads();
+        X::row_sync();
         float2* fm = a.far + ((size_t)b * M + m) * NN;
         X::template r23<+1, 0>(A, tw, [&](V2& v, int ky, int t) {
 #pragma unroll
@@ -357,7 +355,7 @@ __device__ __forceinline__ void path_body(const PathArgs& a) {
       } else {
         // Phi = DFT_-[phi] kept at slot n_dist; then Psi_d = IDFT_-{Phi G_d} per distance
         X::template fwd_pair<-1>(A, tw);
-        __syncthreads();
+        X::row_sync();
         float2* Phi = a.far + (((size_t)b * (nd + 1) + nd) * M + m) * NN;
         X::template r23<-1, 0>(A, tw, [&](V2& v, int ky, int t) {
 #pragma unroll
@@ -378,9 +376,8 @@ __device__ __forceinline__ void path_body(const PathArgs& a) {
               v[i] = cmul(cmul(Phi[ky * N + kx], gy), cmul(__ldg(&hd[kx]), rx[kx]));
             }
           });
-          __syncthreads();
+          X::row_sync();
           X::template inv_pair<+1>(A, tw);
-          __syncthreads();
           float2* fd = a.far + (((size_t)b * (nd + 1) + d) * M + m) * NN;
           float* gId = gI_b + (size_t)d * NN;
           X::template c14<+1, 0, true, false>(A, tw, NoPre(), [&](V1& v, V1&, V1&, int x, int t) {
@@ -507,9 +504,8 @@ __device__ __forceinline__ void path_body(const PathArgs& a) {
           v[i] = cscale(fm[p], sc * gI_b[p]);
         }
       });
-      __syncthreads();
+      X::row_sync();
       X::template inv_pair<-1>(A, tw);
-      __syncthreads();
     } else {
       const float2* Phi = a.far + (((size_t)b * (nd + 1) + nd) * M + m) * NN;
       float2* fb = a.fbar + (size_t)b * NN;
@@ -534,7 +530,7 @@ __device__ __forceinline__ void path_body(const PathArgs& a) {
         });
         __syncthreads();
         X::template fwd_pair<-1>(A, tw);
-        __syncthreads();
+        X::row_sync();
         const float2* hd = a.hd + (size_t)d * N;
         X::template r23<-1, 0>(A, tw, [&](V2& v, int ky, int t) {
           const float2 gy = cmul(__ldg(&hd[ky]), ry[ky]);
@@ -563,9 +559,8 @@ __device__ __forceinline__ void path_body(const PathArgs& a) {
 #pragma unroll
         for (int i = 0; i < RX; ++i) v[i] = cscale(fb[ky * N + t + KXS * i], invNN);
       });
-      __syncthreads();
+      X::row_sync();
       X::template inv_pair<+1>(A, tw);
-      __syncthreads();
     }
 
     for (int s = ncp - 1; s >= 0; --s) {
@@ -586,12 +581,12 @@ __device__ __forceinline__ void path_body(const PathArgs& a) {
         }
         if (own) {
           // park the adjoint field, recompute the segment in shared memory, restore
-          float2* pk = a.park + (size_t)b * N * LD;
-          for (int i = threadIdx.x; i < N * LD; i += NT) pk[i] = A[i];
+          float2* pk = a.park + (size_t)b * NN;
+          __syncthreads();
+          for (int i = threadIdx.x; i < (int)NN; i += NT) pk[i] = A[X::slot(i / N, i % N)];
           __syncthreads();
           recompute(s, sg);
-          for (int i = threadIdx.x; i < N * LD; i += NT) A[i] = pk[i];
-          __syncthreads();
+          for (int i = threadIdx.x; i < (int)NN; i += NT) A[X::slot(i / N, i % N)] = pk[i];
         }
       }
       for (int j = j1; j >= j0; --j) {
@@ -647,7 +642,7 @@ __device__ __forceinline__ void path_body(const PathArgs& a) {
         if (!FAR) continue;
         // far field, j = 0: Q = DFT_-[psibar_0] -> probe and position gradients
         X::template fwd_pair<-1>(A, tw);
-        __syncthreads();
+        X::row_sync();
         const float2* ph = a.phat + (size_t)m * NN;
         float2* q = a.qacc ? a.qacc + ((size_t)b * M + m) * NN : nullptr;
         X::template r23<-1, 0>(A, tw, [&](V2& v, int ky, int t) {
@@ -702,17 +697,17 @@ template <int N, int FAR>
 __device__ __forceinline__ void helper_body(const PathArgs& a) {
   using F = Field<N>;
   using X = PathFFT<N>;
-  constexpr int CY = X::CY, YS = X::YS, RX = X::RX, KXS = X::KXS, LD = F::LD, NT = F::NT;
+  constexpr int CY = X::CY, YS = X::YS, RX = X::RX, KXS = X::KXS, NT = F::NT;
   constexpr size_t NN = (size_t)N * N;
   using V1 = float2[CY];
   using V2 = float2[RX];
   extern __shared__ float2 sm[];
   float2* A = sm;
-  float2* tw = A + N * LD;
-  float2* hy = tw + F::TW_ENTRIES;
+  float2* tw = A + X::FIELD;
+  float2* hy = tw + X::TW;
   float2* hx = hy + N;
   __shared__ int h_task;
-  F::fill_twiddles(tw, a.tw);
+  X::fill_twiddles(tw, a.tw);
   for (int i = threadIdx.x; i < N; i += NT) {
     hy[i] = a.hy[i];
     hx[i] = a.hx[i];
@@ -784,15 +779,14 @@ __device__ __forceinline__ void helper_body(const PathArgs& a) {
       __syncthreads();
       // propagation tail: C2, R1, R23 (H), R4, C3
       X::template fwd_pair<-1>(A, tw);
-      __syncthreads();
+      X::row_sync();
       X::template r23<-1, +1>(A, tw, [&](V2& v, int ky, int t) {
         const float2 h = hy[ky];
 #pragma unroll
         for (int i = 0; i < RX; ++i) v[i] = cmul(cmul(v[i], h), hx[t + KXS * i]);
       });
-      __syncthreads();
+      X::row_sync();
       X::template inv_pair<+1>(A, tw);
-      __syncthreads();
     }
     X::template c14<+1, 0, true, false>(A, tw, NoPre(), [&](V1& v, V1&, V1&, int x, int t) {
 #pragma unroll
@@ -827,10 +821,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Geo<N>::NT, Geo<N>::
   path_body<N, FAR, false, true>(a);
 }
 
-// field + twiddle tables (3N) + hy, hx, ry, rx tables + one double per warp for block reductions
+// field + twiddle tables + hy, hx, ry, rx tables + one double per warp for block reductions
 template <int N>
 constexpr int path_smem_bytes_t() {
-  return (N * (N + 1) + Field<N>::TW_ENTRIES + 4 * N) * (int)sizeof(float2) + (Geo<N>::NT / 32) * (int)sizeof(double);
+  return (PathFFT<N>::FIELD + PathFFT<N>::TW + 4 * N) * (int)sizeof(float2) + (Geo<N>::NT / 32) * (int)sizeof(double);
 }
 
 template <int N, int FAR, bool GAP>

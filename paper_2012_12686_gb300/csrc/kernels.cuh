@@ -47,7 +47,7 @@ struct PathArgs {
   const float2* hd;       // near field: [n_dist][N] factors exp(i pi f^2 / N_F) (unscaled)
   float2* ckpt;           // [B][M][ncp][N*N] checkpoints psi_{j0}
   float2* seg;            // [B][M][cp][N*N] recomputed psi_j of one segment
-  float2* park;           // [B][N*(N+1)] adjoint field parked during a recompute
+  float2* park;           // [B][N*N] adjoint field parked during a recompute
   float2* far;            // [B][M][N*N] detector field (far) or [B][n_dist][M][N*N] (near)
   float* gI;              // [B][N*N] (or [B][n_dist][N*N]) intensity, then dL/dI
   float2* fbar;           // near field: [B][N*N] accumulated Fourier-space adjoint
