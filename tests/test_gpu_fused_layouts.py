@@ -27,30 +27,26 @@ def test_near(N, L, M, B, nd):
     _compare(C.small_case(N=N, L=L, M=M, B=B, loss="lsq", far=False, n_dist=nd, seed=2 + N + L))
 
 
-@pytest.mark.parametrize("N", [64, 128])
-def test_equal_gaps_match_uniform(N):
-    """Equal gaps take the variable-spacing kernel: same stages, same FP64-built tables, so the same
-    values up to the order of the FP64 object-gradient sums."""
+@pytest.mark.parametrize("N,L,M,cp", [(128, 4, 1, 0), (128, 3, 2, 1), (64, 5, 2, 0)])
+def test_variable_spacing(N, L, M, cp):
+    """The variable-spacing instantiation: intensities, object and slice-gap gradients."""
     import torch
+    import oracle
     from paper_2012_12686_gb300.adorym import Engine
-    L = 5
-    case = C.small_case(N=N, L=L, M=1, B=3, loss="poisson", seed=N)
-    p = case["problem"]
+    case = C.small_case(N=N, L=L, M=M, B=2, loss="lsq", cp=cp, seed=31 + N + L)
+    p = dict(case["problem"], gaps=[0.2 + 0.3 * j for j in range(L - 1)])
+    Im = C.measured(dict(case, problem=p)).astype(np.float32)
+    ref = oracle.loss_grad(p, case["delta"], case["beta"], case["probe"], case["pos"], Im, want_gaps=True)
     t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
-    d, b, probe, pos = t(case["delta"]), t(case["beta"]), t(case["probe"].astype(np.complex64)), t(case["pos"])
+    d, b = t(case["delta"]), t(case["beta"])
     eng = Engine(0)
     oid = eng.register_object(d, b)
-    Im = torch.zeros((3, N, N), device="cuda")
-    eng.forward(p, oid, probe, pos, Im)
-    Im = 0.9 * Im + 0.5
-
-    def call(problem):
-        out = [torch.zeros((), dtype=torch.float64, device="cuda"), torch.zeros_like(d), torch.zeros_like(b),
-               torch.zeros_like(probe), torch.zeros_like(pos)]
-        eng.loss_grad(problem, oid, probe, pos, Im, *out)
-        torch.cuda.synchronize()
-        return [x.cpu().numpy() for x in out]
-
-    for x, y in zip(call(p), call(dict(p, gaps=[p["lambda_dz_over_px2"]] * (L - 1)))):
-        assert C.rel(x, y) <= 1e-6
+    gd, gb = torch.zeros_like(d), torch.zeros_like(b)
+    gg, I = torch.zeros(L - 1, device="cuda"), torch.zeros(Im.shape, device="cuda")
+    eng.loss_grad_ext(p, oid, t(case["probe"].astype(np.complex64)), t(case["pos"]), t(Im), g_delta=gd, g_beta=gb,
+                      g_gaps=gg, I_out=I)
+    torch.cuda.synchronize()
+    assert C.rel(I.cpu().numpy(), oracle.forward(p, case["delta"], case["beta"], case["probe"], case["pos"])) <= C.TOL_I
+    for x, y in ((gd, ref[1]), (gb, ref[2]), (gg, ref[-1])):
+        assert C.rel(x.cpu().numpy(), y) <= C.TOL_G
     eng.close()
