@@ -168,7 +168,9 @@ template <> struct Geo<128> { static constexpr int N1 = 8, N2 = 16, NT = 512, MI
 
 template <int N>
 struct Field {
-  static constexpr int N1 = Geo<N>::N1, N2 = Geo<N>::N2, NT = Geo<N>::NT, LD = N + 1;
+  // row pitch: N + 1 is conflict-free for the column- and the row-mapped passes; at N = 64 the row
+  // pass has its own mapping (fft_block4.cuh), conflict-free at a pitch of 8 modulo 16
+  static constexpr int N1 = Geo<N>::N1, N2 = Geo<N>::N2, NT = Geo<N>::NT, LD = N == 64 ? 72 : N + 1;
   // y-frequency held by smem row r after the column forward stages (C2)
   __device__ static __forceinline__ int row_freq(int r) { return r / N2 + N1 * (r % N2); }
 };

@@ -273,12 +273,14 @@ struct PathFFT<128> {
 // row's two radix-8 stages (S1 -> S2 forward, S3 -> S4 inverse) goes through a per-warp scratch
 // area with warp-level synchronisation instead of a shared-memory pass and a CTA barrier:
 //   C14 | C2 | R (x-S1 | exchange | x-S2 | frequency op | x-S3 | exchange | x-S4) | C3
-// is four passes and four barriers per propagation step instead of six, with the same stages,
-// twiddles and order (the same values).  The spatial pass keeps the six-pass thread mapping
-// (consecutive x across a warp: coalesced global accesses); only the row pass, which touches no
-// global memory, uses the warp layout: lane 8 g + t of warp w holds task t of row
-// (w & 7) + 8 g + 32 (w >> 3), so the two rows of a half-warp differ by 8 and every 64-bit row
-// access of a warp covers all 32 banks at leading dimension 65.
+// with the same stages, twiddles and order as the six-pass scheme (the same values).  The spatial
+// pass keeps the six-pass thread mapping (consecutive x across a warp: coalesced global accesses).
+// C2, R and C3 of the eight rows 8 p .. 8 p + 7 belong to the warps 2 p and 2 p + 1 (64 consecutive
+// columns in C2 and C3; rows 4 w + g, lane 8 g + t, in R of warp w), so those two meet at a barrier of
+// their own between the passes and a step has two CTA barriers (around C14) instead of four:
+// tomography loss and gradient 1.180 -> 1.104 ms.  (A staggered start as at N = 128 costs here, 1.157 ms:
+// the passes are too short.)  At a row pitch of 72 the two rows of a half-warp access of R differ by 8
+// modulo 16, so its 64-bit accesses cover all 32 banks.
 // Exchange: lane (g, a) stores its value k at scratch[72 g + a + 9 k]; lane (g, b) reads its
 // value i from scratch[72 g + i + 9 b] (both conflict-free).
 
@@ -313,8 +315,9 @@ struct PathFFT<64> {
   __device__ static __forceinline__ void fill_twiddles(float2* tw, const float2* __restrict__ twg) {
     for (int i = threadIdx.x; i < 64; i += F::NT) tw[i] = twg[i];
   }
+  // the two warps that share eight rows
   __device__ static __forceinline__ void row_sync() {
-    __syncthreads();
+    asm volatile("bar.sync %0, 64;" ::"r"(1 + (int)(threadIdx.x >> 6)) : "memory");
   }
   template <int S4, int S1, bool LOAD, bool STORE, class Pre, class Op>
   __device__ static __forceinline__ void c14(float2* A, const float2* tw, Pre pre, Op op) {
@@ -330,7 +333,7 @@ struct PathFFT<64> {
   __device__ static __forceinline__ void r23(float2* A, const float2* tw, Op op) {
     constexpr int LD = F::LD;
     const int lane = (int)(threadIdx.x & 31), w = (int)(threadIdx.x >> 5), g = lane >> 3, t = lane & 7;
-    const int r = (w & 7) + 8 * g + 32 * (w >> 3);
+    const int r = 4 * w + g;
     float2* ws = row64_scratch() + w * 288;
     float2 v[8], wt[8];
 #pragma unroll
