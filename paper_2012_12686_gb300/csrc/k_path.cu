@@ -76,13 +76,37 @@ __global__ void __launch_bounds__(256) k_qsum(const float2* __restrict__ qacc, f
   }
 }
 
-__global__ void k_gap_final(const double* __restrict__ gapp, int B, int ngap, int parts, float* __restrict__ g) {
-  for (int j = threadIdx.x; j < ngap; j += blockDim.x) {
-    double s = 0.0;
-    for (int b = 0; b < B; ++b)
-      for (int k = 0; k < parts; ++k) s += gapp[((size_t)b * ngap + j) * parts + k];
-    g[j] = (float)s;
+// The same for a batch too small to split: a thread per element, the batch in its own order.
+__global__ void __launch_bounds__(256) k_qsum_few(const float2* __restrict__ qacc, float2* __restrict__ qsum, int B,
+                                                  size_t MNN) {
+  const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
+  if (i >= MNN) return;
+  Kahan sr, si;
+#pragma unroll 4
+  for (int b = 0; b < B; ++b) {
+    const float2 v = __ldg(qacc + (size_t)b * MNN + i);
+    sr.add(v.x);
+    si.add(v.y);
   }
+  qsum[i] = make_float2((float)sr.value(), (float)si.value());
+}
+
+// g_gap[j] = sum of gap j's partials over the positions and column CTAs, one CTA per gap, threads strided
+// over the partials, then a fixed tree.  (Gaps walked by the threads of one CTA, one after the other over
+// the batch, took 40 us for 7 gaps and 100 positions.)
+__global__ void __launch_bounds__(128) k_gap_final(const double* __restrict__ gapp, int B, int ngap, int parts,
+                                                   float* __restrict__ g) {
+  __shared__ double red[4];
+  const int j = blockIdx.x;
+  double s = 0.0;
+#pragma unroll 4
+  for (int i = threadIdx.x; i < B * parts; i += 128)
+    s += gapp[((size_t)(i / parts) * ngap + j) * parts + i % parts];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) g[j] = (float)(((red[0] + red[1]) + red[2]) + red[3]);
 }
 
 // Per-angle position offset of ptychotomography (Sec. 2.3.2): one correction vector shifts every
@@ -111,12 +135,16 @@ cudaError_t launch_offset_sum(const double* gposd, int B, float* g_off, cudaStre
 }
 
 cudaError_t launch_gap_final(const double* gapp, int B, int ngap, int parts, float* g_gap, cudaStream_t s) {
-  (k_gap_final<<<1, 256, 0, s>>>(gapp, B, ngap, parts, g_gap), note_launch());
+  (k_gap_final<<<ngap, 128, 0, s>>>(gapp, B, ngap, parts, g_gap), note_launch());
   return cudaGetLastError();
 }
 
 cudaError_t launch_qsum(const float2* qacc, float2* qsum, int B, size_t MNN, cudaStream_t s) {
-  (k_qsum<<<(unsigned)((MNN + 31) / 32), 256, 0, s>>>(qacc, qsum, B, MNN), note_launch());
+  // up to 8 positions the eight batch chunks of k_qsum hold one value or none (21 us for 2 x 512 x 512)
+  if (B <= 8)
+    (k_qsum_few<<<(unsigned)((MNN + 255) / 256), 256, 0, s>>>(qacc, qsum, B, MNN), note_launch());
+  else
+    (k_qsum<<<(unsigned)((MNN + 31) / 32), 256, 0, s>>>(qacc, qsum, B, MNN), note_launch());
   return cudaGetLastError();
 }
 
@@ -226,9 +254,7 @@ template <int N, int FAR>
 static cudaError_t launch_probe_grad_t(int M, int B, const float2* qacc, float2* qsum, float2* g, const float2* tw,
                                        const double* lossp, double inv_npix, double* loss_out, cudaStream_t s) {
   const size_t MNN = (size_t)M * N * N;
-  if (g) {
-    (k_qsum<<<(unsigned)((MNN + 31) / 32), 256, 0, s>>>(qacc, qsum, B, MNN), note_launch());
-  }
+  if (g) launch_qsum(qacc, qsum, B, MNN, s);
   const int smem = probe_smem_bytes<N>();
   (k_probe_grad<N, FAR><<<M, Geo<N>::NT, smem, s>>>(qsum, g, tw, lossp, B, inv_npix, loss_out), note_launch());
   return cudaGetLastError();
