@@ -1,5 +1,6 @@
 // C ABI entry points: context, object registration, validation, workspace planning, FP64-built
 // tables, host-argument staging and the launch sequence of one loss/gradient call.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -109,9 +110,11 @@ int make_plan(const adorym_problem& p, bool adj, int grads, bool want_loss, Plan
       q.off_seg = take(B * M * q.cp * NN * f2);
       q.off_qacc = take(B * M * NN * f2);
       q.off_qsum = take(M * NN * f2);
-      q.off_posp = take(B * q.nd * (N / (N == 256 ? 64 : N == 512 ? 32 : 16)) * 3 * sizeof(double));
     }
-    q.off_tmp = take(M * NN * f2);
+    // the position partials live between the probe transform and the probe-gradient transform, which
+    // are the users of tmp: one region for both
+    q.off_tmp = take(std::max(M * NN * f2, adj ? B * q.nd * twopass_columns(p.N) * 3 * sizeof(double) : 0));
+    q.off_posp = q.off_tmp;
     q.off_far = take(B * (q.far ? 1 : q.nd + 1) * M * NN * f2);
     q.off_gI = take(B * q.nd * NN * sizeof(float));
     q.off_lossp = take(B * q.nd * (NN / 1024) * sizeof(double));
@@ -139,7 +142,7 @@ int make_plan(const adorym_problem& p, bool adj, int grads, bool want_loss, Plan
     q.off_s_goff = take(2 * sizeof(float));
   }
   if (q.want_gaps) {
-    const int parts = two_pass(p.N) ? (int)(N / (N == 256 ? 32 : N == 512 ? 16 : 8)) : 1;
+    const int parts = two_pass(p.N) ? twopass_columns(p.N) : 1;
     q.off_spck = take(B * M * q.ncp * NN * f2);
     q.off_spseg = take(B * M * q.cp * NN * f2);
     q.off_gapp = take(B * (size_t)(p.L - 1) * parts * sizeof(double));

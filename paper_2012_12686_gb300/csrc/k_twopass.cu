@@ -14,7 +14,9 @@
 // x-transform) + column kernel (forward y-transform, propagator, inverse y-transform).  The
 // row tile uses a skewed shared-memory layout (one pad element after every N2 elements), which
 // keeps both the strided and the contiguous stage accesses free of bank conflicts with the
-// lane index on the x digit, so every global access is coalesced.  The column tile is brought in
+// lane index on the x digit, so every global access is coalesced; a warp has its rows through all three
+// stages, so a row kernel has no CTA barrier after its tables.  The kernels of a sequence are chained by
+// programmatic dependent launch (Seq).  The column tile is brought in
 // by TMA (a 2-D tensor map over the field buffer, completion on an mbarrier) and lands in the
 // [row][column] layout the first in-place stage reads.  With one probe mode and measured data the
 // detector pass also forms the loss term and the adjoint seed.  Loss and position-gradient
@@ -33,21 +35,51 @@ namespace adorym {
 
 template <int N>
 struct Geo2;
-// RB rows per row-kernel CTA, CW columns per column-kernel CTA; 256 threads, tiles of ~64 KB so
-// two CTAs share an SM and one CTA's loads overlap the other's transforms
-template <> struct Geo2<256>  { static constexpr int N1 = 16, N2 = 16, RB = 16, CW = 32; };
+// RB rows per row-kernel CTA, CW columns per column-kernel CTA; 256 threads.  N >= 512: tiles of 64 KB, two
+// CTAs per SM, one's loads under the other's transforms.  N = 256: column tiles of 32 KB (a 128-byte
+// row of a TMA box), one task per thread in every stage, so that 64 registers hold it and four CTAs share
+// an SM: 64 positions are 1024 CTAs of 608 slots, where 64 KB tiles at three per SM were 512 of 456 and
+// the second wave was an eighth full (64 x 8 loss and gradient 1126 -> 1057 us, 128 x 32 7505 -> 7094).
+template <> struct Geo2<256>  { static constexpr int N1 = 16, N2 = 16, RB = 16, CW = 16; };
 template <> struct Geo2<512>  { static constexpr int N1 = 16, N2 = 32, RB = 16, CW = 16; };
 template <> struct Geo2<1024> { static constexpr int N1 = 32, N2 = 32, RB = 8, CW = 8; };
 constexpr int NT2 = 256;
 
+// Twiddles between the two stages of a transform, by stage and contiguous in the task index:
+// tw[k N1 + t] = W_N^(t k) after a DFT_N2 (S3, task t < N1), and the same with N2 in the place of N1
+// after a DFT_N1 (S1); one table where N1 = N2.  The lanes of a row pass run over t: read at t k from
+// the table of W_N^m they met gcd(k, 16) to a bank (160 instead of 62 wavefronts per warp and stage at
+// N = 1024, more than the data's exchange).
+template <int N>
+struct Tw2 {
+  static constexpr int N1 = Geo2<N>::N1, N2 = Geo2<N>::N2;
+  static constexpr int SIZE = N1 == N2 ? N : 2 * N;
+  __device__ static __forceinline__ void fill(float2* tw, const float2* __restrict__ twg) {
+    for (int i = threadIdx.x; i < N; i += NT2) {
+      tw[i] = __ldg(twg + (i / N1) * (i % N1));
+      if (N1 != N2) tw[N + i] = __ldg(twg + (i / N2) * (i % N2));
+    }
+  }
+  // v[k] *= W_N^(S t k) after a DFT_R
+  template <int S, int R>
+  __device__ static __forceinline__ void apply(float2 (&v)[R], const float2* __restrict__ tw, int t) {
+    const float2* p = tw + (R == N2 ? 0 : N) + t;   // (N1 == N2: R == N2 either way)
+#pragma unroll
+    for (int k = 1; k < R; ++k) {
+      const float2 w = p[k * (N / R)];
+      v[k] = S < 0 ? cmul(v[k], w) : cmulc(v[k], w);
+    }
+  }
+};
+
 template <int N>
 constexpr int row_smem_bytes() {
-  return Geo2<N>::RB * (N + Geo2<N>::N1) * (int)sizeof(float2) + N * (int)sizeof(float2) + 64 * 8;
+  return Geo2<N>::RB * (N + Geo2<N>::N1) * (int)sizeof(float2) + Tw2<N>::SIZE * (int)sizeof(float2) + 64 * 8;
 }
-// column tile + tw, ry, hy tables + 64 doubles of reduction scratch + one mbarrier (TMA staging)
+// column tile + twiddles, ry, hy tables + 64 doubles of reduction scratch + one mbarrier (TMA staging)
 template <int N>
 constexpr int col_smem_bytes() {
-  return N * Geo2<N>::CW * (int)sizeof(float2) + 3 * N * (int)sizeof(float2) + 64 * 8 + 16;
+  return (N * Geo2<N>::CW + Tw2<N>::SIZE + 2 * N) * (int)sizeof(float2) + 64 * 8 + 16;
 }
 
 // R_NEAR_DSEED / C_FAR_SEED (one probe mode with measured data; the _P forms for the Poisson loss,
@@ -57,21 +89,17 @@ constexpr int col_smem_bytes() {
 enum RowMode { R_FWD, R_RC_FIRST, R_RC, R_ADJ, R_NEAR_DET, R_NEAR_SEED, R_PHAT, R_PG_OUT, R_NEAR_DSEED, R_NEAR_DSEED_P };
 enum ColMode { C_PROP, C_PROP_ADJ, C_PSI0, C_FAR, C_SEED, C_Q, C_PHAT, C_PG, C_NEAR_PHI, C_NEAR_Q, C_FAR_SEED, C_FAR_SEED_P };
 
-// Resident CTAs per SM the register budget of a row / column kernel is sized for.  At N = 256 the
-// slice-step kernels of the forward and recompute sweeps and the propagation column kernels fit
-// three per SM without spilling (80 registers; shared memory 37 / 71 KB per CTA), which puts more
-// loads in flight in these latency-bound passes; the other modes keep two (their larger register
-// sets would spill).  ADORYM_TP256_OCC3 = 0 keeps two everywhere.
-#ifndef ADORYM_TP256_OCC3
-#define ADORYM_TP256_OCC3 1
-#endif
+// Resident CTAs per SM the register budget of a row / column kernel is sized for.  N = 256: the
+// propagation columns fit four (64 registers, no spills), the other columns and the row kernels of the
+// forward and recompute sweeps three (80); the adjoint rows keep two (at three they spill, and gain
+// nothing), as do the 32-value stages of N >= 512.
 template <int N, int MODE>
 constexpr int row_minb() {
-  return (ADORYM_TP256_OCC3 && N == 256 && (MODE == R_FWD || MODE == R_RC_FIRST)) ? 3 : 2;
+  return N == 256 && (MODE == R_FWD || MODE == R_RC_FIRST || MODE == R_RC) ? 3 : 2;
 }
 template <int N, int MODE>
 constexpr int col_minb() {
-  return (ADORYM_TP256_OCC3 && N == 256 && (MODE == C_PROP || MODE == C_PROP_ADJ)) ? 3 : 2;
+  return N != 256 ? 2 : (MODE == C_PROP || MODE == C_PROP_ADJ) ? 4 : 3;
 }
 
 __device__ __forceinline__ float freqf(int k, int N) { return (float)(k <= (N - 1) / 2 ? k : k - N) / (float)N; }
@@ -187,6 +215,15 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, i
       : "memory");
 }
 
+// Programmatic dependent launch: the next kernel of the sequence may start its CTAs as soon as all of
+// this one's have started, and runs its prologue (tables, transmission; nothing the sequence writes)
+// until `after_previous`, which returns once the kernel before it has completed and its writes are
+// visible.  Every CTA calls both, so a kernel that has completed implies all before it.  What the
+// sequence itself writes is read with __ldcg (L2): not invariant to the compiler, and never from an L1
+// line that an earlier kernel of the chain left behind.
+__device__ __forceinline__ void allow_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ============================================================================ row kernel
 template <int N, int MODE>
 __global__ void __launch_bounds__(NT2, row_minb<N, MODE>()) k_row(const TPArgs a) {
@@ -195,9 +232,13 @@ __global__ void __launch_bounds__(NT2, row_minb<N, MODE>()) k_row(const TPArgs a
   extern __shared__ float2 sm[];
   float2* A = sm;
   float2* tw = A + RB * LDR;
-  double* red = reinterpret_cast<double*>(tw + N);
+  double* red = reinterpret_cast<double*>(tw + Tw2<N>::SIZE);
   auto idx = [](int r, int p) { return r * LDR + p + p / N2; };
-  for (int i = threadIdx.x; i < N; i += NT2) tw[i] = a.tw[i];
+  constexpr int RPW = RB / (NT2 / 32);   // rows per warp: a warp has its rows through all three stages
+  static_assert(RPW * N1 == 32 && RPW * N2 % 32 == 0, "one S3 / S2 task per lane");
+  const int lane = (int)(threadIdx.x & 31), rw = (int)(threadIdx.x >> 5) * RPW;
+  allow_next();
+  Tw2<N>::fill(tw, a.tw);
 
   const int r0 = blockIdx.x * RB;
   const int f = blockIdx.y;                         // position / problem b (or probe mode m)
@@ -242,28 +283,67 @@ __global__ void __launch_bounds__(NT2, row_minb<N, MODE>()) k_row(const TPArgs a
     src = a.tmp + (size_t)f * NN;
     out = 0;
   }
+  after_previous();
   __syncthreads();
 
   // ---- stage IN: S3 from global (natural kx = t + N1 i)
+  const int t1 = lane % N1, r1 = rw + lane / N1;   // this lane's S3 / S2 task
   if (in_freq) {
-    for (int tau = threadIdx.x; tau < RB * N1; tau += NT2) {
-      const int t = tau % N1, r = tau / N1;
+    {
+      const int t = t1, r = r1;
       const float2* row = src + (size_t)(r0 + r) * N;
       float2 v[N2];
 #pragma unroll
-      for (int i = 0; i < N2; ++i) v[i] = row[t + N1 * i];
-      if (si < 0) { dft<N2, -1>(v); twiddle<-1>(v, tw, t); }
-      else { dft<N2, +1>(v); twiddle<+1>(v, tw, t); }
+      for (int i = 0; i < N2; ++i) v[i] = __ldcg(row + t + N1 * i);
+      if (si < 0) { dft<N2, -1>(v); Tw2<N>::template apply<-1>(v, tw, t); }
+      else { dft<N2, +1>(v); Tw2<N>::template apply<+1>(v, tw, t); }
 #pragma unroll
       for (int k = 0; k < N2; ++k) A[idx(r, N2 * t + k)] = v[k];
     }
-    __syncthreads();
+    __syncwarp();
   }
   // ---- stage MID: S4 -> natural x = N2 k + t -> op -> S1
   Kahan lacc;   // R_NEAR_DSEED: loss terms of this thread's pixels
-  for (int tau = threadIdx.x; tau < RB * N2; tau += NT2) {
-    const int t = tau % N2, r = tau / N2;
+  for (int tau = lane; tau < RPW * N2; tau += 32) {
+    const int t = tau % N2, r = rw + tau / N2;
     const int y = r0 + r;
+    // transmission (and psi, gradient) values come in chunks of CH, a chunk's loads issued ahead of the
+    // x-S4 or of the chunk before it, and ahead of any store
+    constexpr bool ADJ = MODE == R_ADJ, MODULATES = ADJ || MODE == R_FWD || MODE == R_RC_FIRST || MODE == R_RC;
+    constexpr int CH = ADJ ? 4 : 8;
+    int p0y = 0, p0x = 0;
+    if (MODULATES && FAR) {
+      p0y = patch_corner(a.pos[2 * b]);
+      p0x = patch_corner(a.pos[2 * b + 1]);
+    }
+    const int gz = FAR ? j : b * a.L + j, gy = p0y + y;
+    const bool row_in = gy >= 0 && gy < a.Ly;
+    const size_t orow = ((size_t)gz * a.Ly + gy) * a.Lx + p0x + t;   // voxel of pixel k: orow + N2 k
+    const float2* psrc = nullptr;
+    if (ADJ)
+      psrc = (j == a.j0) ? a.ckpt + (((size_t)b * a.M + m) * a.ncp + a.s) * NN
+                         : a.seg + (((size_t)b * a.M + m) * a.cp + (j - a.j0)) * NN;
+    float2 Tv[2][CH], pv[2][ADJ ? CH : 1];
+    float gdv[2][ADJ ? CH : 1], gbv[2][ADJ ? CH : 1];
+    auto inside = [&](int k) {
+      const int gx = p0x + N2 * k + t;
+      return row_in && gx >= 0 && gx < a.Lx;
+    };
+    auto load_chunk = [&](int h, int k0) {
+#pragma unroll
+      for (int c = 0; c < CH; ++c) {
+        const int k = k0 + c;
+        Tv[h][c] = inside(k) ? __ldg(a.T + orow + N2 * k) : make_float2(1.f, 0.f);
+        if (ADJ) {
+          pv[h][ADJ ? c : 0] = __ldcg(psrc + (size_t)y * N + N2 * k + t);
+          if (a.gdf) {
+            gdv[h][ADJ ? c : 0] = a.gdf[orow + N2 * k];
+            gbv[h][ADJ ? c : 0] = a.gbf[orow + N2 * k];
+          }
+        }
+      }
+    };
+    if (MODULATES) load_chunk(0, 0);
     float2 v[N1];
     if (in_freq) {
 #pragma unroll
@@ -272,96 +352,43 @@ __global__ void __launch_bounds__(NT2, row_minb<N, MODE>()) k_row(const TPArgs a
       else dft<N1, +1>(v);
     } else {
 #pragma unroll
-      for (int k = 0; k < N1; ++k) v[k] = src[(size_t)y * N + N2 * k + t];
+      for (int k = 0; k < N1; ++k) v[k] = __ldcg(src + (size_t)y * N + N2 * k + t);
     }
     // spatial ops; x = N2 k + t
-    if (MODE == R_FWD || MODE == R_RC_FIRST || MODE == R_RC) {
-      int p0y = 0, p0x = 0, gz = FAR ? j : b * a.L + j;
-      if (FAR) {
-        p0y = patch_corner(a.pos[2 * b]);
-        p0x = patch_corner(a.pos[2 * b + 1]);
+    if (MODULATES) {
+      float2* keep = nullptr;   // psi_j: checkpoint, segment slot or nowhere
+      if (MODE == R_FWD && a.adj) {
+        if (j % a.cp == 0) keep = a.ckpt + (((size_t)b * a.M + m) * a.ncp + j / a.cp) * NN;
+        else if (j > (a.ncp - 1) * a.cp) keep = a.seg + (((size_t)b * a.M + m) * a.cp + (j - (a.ncp - 1) * a.cp)) * NN;
+      } else if (MODE == R_RC) {
+        keep = a.seg + (((size_t)b * a.M + m) * a.cp + (j - a.j0)) * NN;
       }
-      const int gy = p0y + y;
-      const bool row_in = gy >= 0 && gy < a.Ly;
-      float2* ck = a.ckpt + ((size_t)b * a.M + m) * a.ncp * NN;
-      float2* sg = a.seg + ((size_t)b * a.M + m) * a.cp * NN;
-      // transmission loads in chunks ahead of the checkpoint / segment stores
-      constexpr int CH = N1 >= 32 ? 8 : N1;
 #pragma unroll
       for (int k0 = 0; k0 < N1; k0 += CH) {
-        float2 Tv[CH];
-#pragma unroll
-        for (int c = 0; c < CH; ++c) {
-          const int gx = p0x + N2 * (k0 + c) + t;
-          const bool inb = row_in && gx >= 0 && gx < a.Lx;
-          Tv[c] = inb ? __ldg(a.T + ((size_t)gz * a.Ly + gy) * a.Lx + gx) : make_float2(1.f, 0.f);
-        }
+        const int h = (k0 / CH) & 1;
+        if (k0 + CH < N1) load_chunk(1 - h, k0 + CH);
 #pragma unroll
         for (int c = 0; c < CH; ++c) {
           const int k = k0 + c;
-          const float2 T = Tv[c];
           const size_t px = (size_t)y * N + N2 * k + t;
-          if (MODE == R_FWD) {
-            if (a.adj) {
-              if (j % a.cp == 0) ck[(size_t)(j / a.cp) * NN + px] = v[k];
-              else if (j > (a.ncp - 1) * a.cp) sg[(size_t)(j - (a.ncp - 1) * a.cp) * NN + px] = v[k];
-            }
-            v[k] = cmul(v[k], T);
-          } else if (MODE == R_RC_FIRST) {
-            v[k] = cmul(v[k], T);
-          } else if (MODE == R_RC) {
-            sg[(size_t)(j - a.j0) * NN + px] = v[k];
-            v[k] = cmul(v[k], T);
+          if (!ADJ) {
+            if (keep) keep[px] = v[k];
+            v[k] = cmul(v[k], Tv[h][c]);
+            continue;
           }
-        }
-      }
-    }
-    if (MODE == R_ADJ) {
-      int p0y = 0, p0x = 0, gz = FAR ? j : b * a.L + j;
-      if (FAR) {
-        p0y = patch_corner(a.pos[2 * b]);
-        p0x = patch_corner(a.pos[2 * b + 1]);
-      }
-      const int gy = p0y + y;
-      const bool row_in = gy >= 0 && gy < a.Ly;
-      const float2* psrc = (j == a.j0) ? a.ckpt + (((size_t)b * a.M + m) * a.ncp + a.s) * NN
-                                       : a.seg + (((size_t)b * a.M + m) * a.cp + (j - a.j0)) * NN;
-      // chunks of CH pixels: all loads of a chunk (T, psi and, in place, the gradient values)
-      // are issued before any of its stores, so they are in flight together
-      constexpr int CH = N1 >= 32 ? 4 : 8;
-#pragma unroll
-      for (int k0 = 0; k0 < N1; k0 += CH) {
-        float2 Tv[CH], pv[CH];
-        float gdv[CH], gbv[CH];
-#pragma unroll
-        for (int c = 0; c < CH; ++c) {
-          const int x = N2 * (k0 + c) + t, gx = p0x + x;
-          const bool inb = row_in && gx >= 0 && gx < a.Lx;
-          const size_t o = ((size_t)gz * a.Ly + gy) * a.Lx + gx;
-          Tv[c] = inb ? __ldg(a.T + o) : make_float2(1.f, 0.f);
-          pv[c] = __ldg(psrc + (size_t)y * N + x);
-          if (a.gdf) {
-            gdv[c] = a.gdf[o];
-            gbv[c] = a.gbf[o];
-          }
-        }
-#pragma unroll
-        for (int c = 0; c < CH; ++c) {
-          const int k = k0 + c, x = N2 * k + t, gx = p0x + x;
-          const bool inb = row_in && gx >= 0 && gx < a.Lx;
-          const size_t o = ((size_t)gz * a.Ly + gy) * a.Lx + gx;
-          const float2 pbar = cmulc(v[k], Tv[c]);
-          const float2 z = cmulc(pbar, pv[c]);
+          const float2 pbar = cmulc(v[k], Tv[h][c]);
+          const float2 z = cmulc(pbar, pv[h][ADJ ? c : 0]);
+          const size_t o = orow + N2 * k;
           if (a.gdf) {
             // near field, one mode: this thread owns the voxel for the whole call
-            a.gdf[o] = gdv[c] + a.kdz * z.y;
-            a.gbf[o] = gbv[c] - a.kdz * z.x;
-          } else if (a.gd && inb) {
+            a.gdf[o] = gdv[h][ADJ ? c : 0] + a.kdz * z.y;
+            a.gbf[o] = gbv[h][ADJ ? c : 0] - a.kdz * z.x;
+          } else if (a.gd && inside(k)) {
             atomicAdd(a.gd + o, f32_to_f64(a.kdz * z.y));
             atomicAdd(a.gb + o, f32_to_f64(-a.kdz * z.x));
           }
           v[k] = pbar;
-          if (!FAR && j == 0 && a.qacc) a.qacc[fo + (size_t)y * N + x] = pbar;
+          if (!FAR && j == 0 && a.qacc) a.qacc[fo + px] = pbar;
         }
       }
     } else if (MODE == R_NEAR_DET) {
@@ -370,12 +397,12 @@ __global__ void __launch_bounds__(NT2, row_minb<N, MODE>()) k_row(const TPArgs a
       for (int k = 0; k < N1; ++k) {
         const size_t px = (size_t)y * N + N2 * k + t;
         const float I = fmaf(v[k].x, v[k].x, v[k].y * v[k].y);
-        g[px] = (m == 0) ? I : g[px] + I;
+        g[px] = (m == 0) ? I : __ldcg(g + px) + I;
       }
     } else if (MODE == R_NEAR_SEED) {
       const float* g = a.gI + ((size_t)b * a.nd + a.d) * NN;
 #pragma unroll
-      for (int k = 0; k < N1; ++k) v[k] = cscale(v[k], 2.0f * g[(size_t)y * N + N2 * k + t]);
+      for (int k = 0; k < N1; ++k) v[k] = cscale(v[k], 2.0f * __ldcg(g + (size_t)y * N + N2 * k + t));
     } else if (MODE == R_NEAR_DSEED || MODE == R_NEAR_DSEED_P) {
       const size_t pb = ((size_t)b * a.nd + a.d) * NN + (size_t)y * N + t;
       const float sc = 2.0f * (float)a.inv_npix;
@@ -399,8 +426,8 @@ __global__ void __launch_bounds__(NT2, row_minb<N, MODE>()) k_row(const TPArgs a
       }
     }
     if (out == 1) {
-      if (so < 0) { dft<N1, -1>(v); twiddle<-1>(v, tw, t); }
-      else { dft<N1, +1>(v); twiddle<+1>(v, tw, t); }
+      if (so < 0) { dft<N1, -1>(v); Tw2<N>::template apply<-1>(v, tw, t); }
+      else { dft<N1, +1>(v); Tw2<N>::template apply<+1>(v, tw, t); }
 #pragma unroll
       for (int k = 0; k < N1; ++k) A[idx(r, N2 * k + t)] = v[k];
     } else if (out == 2) {
@@ -413,10 +440,10 @@ __global__ void __launch_bounds__(NT2, row_minb<N, MODE>()) k_row(const TPArgs a
     if (threadIdx.x == 0) a.lossp[((size_t)b * a.nd + a.d) * gridDim.x + blockIdx.x] = ls;
   }
   if (out != 1) return;
-  __syncthreads();
+  __syncwarp();
   // ---- stage OUT: S2 to global (natural kx = t + N1 i)
-  for (int tau = threadIdx.x; tau < RB * N1; tau += NT2) {
-    const int t = tau % N1, r = tau / N1;
+  {
+    const int t = t1, r = r1;
     float2 v[N2];
 #pragma unroll
     for (int i = 0; i < N2; ++i) v[i] = A[idx(r, N2 * t + i)];
@@ -437,7 +464,7 @@ __global__ void __launch_bounds__(NT2, col_minb<N, MODE>()) k_col(const __grid_c
   extern __shared__ __align__(128) float2 sm[];
   float2* C = sm;
   float2* tw = C + N * CW;
-  float2* ry = tw + N;
+  float2* ry = tw + Tw2<N>::SIZE;
   float2* hy = ry + N;                // hy (far: propagator / near: detector factor of distance d)
   double* red = reinterpret_cast<double*>(hy + N);
   uint64_t* bar = reinterpret_cast<uint64_t*>(red + 64);
@@ -453,10 +480,9 @@ __global__ void __launch_bounds__(NT2, col_minb<N, MODE>()) k_col(const __grid_c
   const int gap = (MODE == C_PROP_ADJ) ? a.j - 1 : a.j;
   const float2* hysrc = (a.hyj && (MODE == C_PROP || MODE == C_PROP_ADJ)) ? a.hyj + (size_t)gap * N : a.hy;
   const float2* hxsrc = (a.hxj && (MODE == C_PROP || MODE == C_PROP_ADJ)) ? a.hxj + (size_t)gap * N : a.hx;
-  for (int i = threadIdx.x; i < N; i += NT2) {
-    tw[i] = a.tw[i];
-    hy[i] = hysrc[i];
-  }
+  allow_next();
+  Tw2<N>::fill(tw, a.tw);
+  for (int i = threadIdx.x; i < N; i += NT2) hy[i] = hysrc[i];
   double dry = 0.0, drx = 0.0;
   if (FAR && (MODE == C_PSI0 || MODE == C_Q)) {
     const double py = a.pos[2 * b], px = a.pos[2 * b + 1];
@@ -464,6 +490,7 @@ __global__ void __launch_bounds__(NT2, col_minb<N, MODE>()) k_col(const __grid_c
     drx = px - floor(px + 0.5);
     for (int i = threadIdx.x; i < N; i += NT2) ry[i] = shift_ramp((float)dry, i, N);
   }
+  after_previous();
   __syncthreads();
 
   // tensor map and first row of the field at src (a whole number of rows into FA, FR, far or tmp)
@@ -507,8 +534,8 @@ __global__ void __launch_bounds__(NT2, col_minb<N, MODE>()) k_col(const __grid_c
         float2 v[N1];
 #pragma unroll
         for (int i = 0; i < N1; ++i) v[i] = C[(N2 * i + t) * CW + c];
-        if (sgn < 0) { dft<N1, -1>(v); twiddle<-1>(v, tw, t); }
-        else { dft<N1, +1>(v); twiddle<+1>(v, tw, t); }
+        if (sgn < 0) { dft<N1, -1>(v); Tw2<N>::template apply<-1>(v, tw, t); }
+        else { dft<N1, +1>(v); Tw2<N>::template apply<+1>(v, tw, t); }
 #pragma unroll
         for (int k = 0; k < N1; ++k) C[(N2 * k + t) * CW + c] = v[k];
       }
@@ -518,9 +545,9 @@ __global__ void __launch_bounds__(NT2, col_minb<N, MODE>()) k_col(const __grid_c
       const int c = tau % CW, t = tau / CW;
       float2 v[N1];
 #pragma unroll
-      for (int i = 0; i < N1; ++i) v[i] = src[(size_t)(N2 * i + t) * N + p0 + c];
-      if (sgn < 0) { dft<N1, -1>(v); twiddle<-1>(v, tw, t); }
-      else { dft<N1, +1>(v); twiddle<+1>(v, tw, t); }
+      for (int i = 0; i < N1; ++i) v[i] = __ldcg(src + (size_t)(N2 * i + t) * N + p0 + c);
+      if (sgn < 0) { dft<N1, -1>(v); Tw2<N>::template apply<-1>(v, tw, t); }
+      else { dft<N1, +1>(v); Tw2<N>::template apply<+1>(v, tw, t); }
 #pragma unroll
       for (int k = 0; k < N1; ++k) C[(N2 * k + t) * CW + c] = v[k];
     }
@@ -541,8 +568,8 @@ __global__ void __launch_bounds__(NT2, col_minb<N, MODE>()) k_col(const __grid_c
   };
   // S3 of registers -> smem
   auto s3_store = [&](float2 (&v)[N2], int c, int t, int sgn) {
-    if (sgn < 0) { dft<N2, -1>(v); twiddle<-1>(v, tw, t); }
-    else { dft<N2, +1>(v); twiddle<+1>(v, tw, t); }
+    if (sgn < 0) { dft<N2, -1>(v); Tw2<N>::template apply<-1>(v, tw, t); }
+    else { dft<N2, +1>(v); Tw2<N>::template apply<+1>(v, tw, t); }
 #pragma unroll
     for (int k = 0; k < N2; ++k) C[(N2 * t + k) * CW + c] = v[k];
   };
@@ -580,7 +607,7 @@ __global__ void __launch_bounds__(NT2, col_minb<N, MODE>()) k_col(const __grid_c
         } else {
           if (si) {
             const float fy = freqf(ky, N);
-            gs += (fy * fy + fx * fx) * cmulc(si[(size_t)ky * N + kx], v[i]).y;
+            gs += (fy * fy + fx * fx) * cmulc(__ldcg(si + (size_t)ky * N + kx), v[i]).y;
           }
           v[i] = cmulc(v[i], h);
         }
@@ -609,7 +636,7 @@ __global__ void __launch_bounds__(NT2, col_minb<N, MODE>()) k_col(const __grid_c
 #pragma unroll
         for (int i = 0; i < N2; ++i) {
           const int ky = t + N1 * i;
-          v[i] = cmul(cmul(ph[(size_t)ky * N + kx], ry[ky]), rx);
+          v[i] = cmul(cmul(__ldcg(ph + (size_t)ky * N + kx), ry[ky]), rx);
         }
       } else if (MODE == C_SEED) {
         const float2* fm = a.far + fo;
@@ -618,12 +645,12 @@ __global__ void __launch_bounds__(NT2, col_minb<N, MODE>()) k_col(const __grid_c
 #pragma unroll
         for (int i = 0; i < N2; ++i) {
           const size_t p = (size_t)(t + N1 * i) * N + kx;
-          v[i] = cscale(fm[p], sc * g[p]);
+          v[i] = cscale(__ldcg(fm + p), sc * __ldcg(g + p));
         }
       } else {   // C_PG: qsum / N^2
         const float2* q = a.qsum + (size_t)f * NN;
 #pragma unroll
-        for (int i = 0; i < N2; ++i) v[i] = cscale(q[(size_t)(t + N1 * i) * N + kx], 1.0f / (float)NN);
+        for (int i = 0; i < N2; ++i) v[i] = cscale(__ldcg(q + (size_t)(t + N1 * i) * N + kx), 1.0f / (float)NN);
       }
       s3_store(v, c, t, MODE == C_SEED ? -1 : +1);
     }
@@ -651,7 +678,7 @@ __global__ void __launch_bounds__(NT2, col_minb<N, MODE>()) k_col(const __grid_c
           const float2 P = cscale(v[i], invN);
           fm[p] = P;
           const float I = fmaf(P.x, P.x, P.y * P.y);
-          g[p] = (m == 0) ? I : g[p] + I;
+          g[p] = (m == 0) ? I : __ldcg(g + p) + I;
         }
       } else if (MODE == C_PHAT) {
         float2* o = a.phat_w + (size_t)f * NN;
@@ -667,7 +694,7 @@ __global__ void __launch_bounds__(NT2, col_minb<N, MODE>()) k_col(const __grid_c
           const int ky = t + N1 * i;
           const size_t p = (size_t)ky * N + kx;
           const float2 r = cmul(ry[ky], rx);
-          const float2 base = cmul(cconj(v[i]), cmul(ph[p], r));
+          const float2 base = cmul(cconj(v[i]), cmul(__ldcg(ph + p), r));
           ay += freqf(ky, N) * base.y;
           ax += fx * base.y;
           if (q) q[p] = cmulc(v[i], r);
@@ -772,7 +799,7 @@ __global__ void __launch_bounds__(NT2, col_minb<N, MODE>()) k_col(const __grid_c
 #pragma unroll
           for (int e = 0; e < CH; ++e) {
             const size_t p = (size_t)(t + N1 * (i0 + e)) * N + kx;
-            ph[e] = __ldg(Phi + p);
+            ph[e] = __ldcg(Phi + p);
             ac[e] = (d == 0) ? make_float2(0.f, 0.f) : acc[p];
           }
 #pragma unroll
@@ -834,48 +861,49 @@ __global__ void __launch_bounds__(256) k_loss2(const TPArgs a) {
   if (threadIdx.x == 0) a.lossp[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = s;
 }
 
-// loss: all threads over the partials, fixed split and order; shift / Fresnel-number gradients: one
-// warp per (problem, distance), lanes over the column-CTA partials, fixed shuffle tree
-__global__ void __launch_bounds__(1024) k_final2(const TPArgs a, int nloss, int ncolblk) {
-  __shared__ double red[32];
-  if (a.loss_out) {
-    const int chunk = (nloss + blockDim.x - 1) / blockDim.x;
+// Block 0: the loss, all threads over the partials in a fixed split and order.  Block 1 + q: shift and
+// Fresnel-number gradients of (problem, distance) q from its column-CTA partials.  One SM adds about two
+// FP64 values a clock, so all of it in one CTA of 32 warps took 20 us (holography) to 35 us (128 positions).
+__global__ void __launch_bounds__(128) k_final2(const TPArgs a, int nloss, int ncolblk) {
+  __shared__ double red[12];
+  if (blockIdx.x == 0) {
+    if (!a.loss_out) return;
     double acc = 0.0;
-    for (int i = threadIdx.x * chunk; i < min(nloss, (int)(threadIdx.x + 1) * chunk); ++i) acc += a.lossp[i];
+#pragma unroll 4
+    for (int i = threadIdx.x; i < nloss; i += 128) acc += a.lossp[i];
     const double s = block_sum2(acc, red);
     if (threadIdx.x == 0) *a.loss_out = s * a.inv_npix;
+    return;
   }
-  if (a.posp && (a.gpos || a.gposd || a.gnf)) {
-    const double pi = 3.14159265358979323846, NN = (double)a.N * a.N, sc = 2.0 * pi / NN;
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int q = w; q < a.B * a.nd; q += nw) {
-      double sy = 0.0, sx = 0.0, sn = 0.0;
-      for (int k = l; k < ncolblk; k += 32) {
-        const double* pp = a.posp + ((size_t)q * ncolblk + k) * 3;
-        sy += pp[0];
-        sx += pp[1];
-        sn += pp[2];
-      }
+  const int q = (int)blockIdx.x - 1;
+  double v[3] = {0.0, 0.0, 0.0};
+  for (int k = threadIdx.x; k < ncolblk; k += 128) {
+    const double* pp = a.posp + ((size_t)q * ncolblk + k) * 3;
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        sy += __shfl_xor_sync(0xffffffffu, sy, o);
-        sx += __shfl_xor_sync(0xffffffffu, sx, o);
-        sn += __shfl_xor_sync(0xffffffffu, sn, o);
-      }
-      if (l == 0) {
-        if (a.gpos) {
-          a.gpos[2 * q] = (float)(sc * sy);
-          a.gpos[2 * q + 1] = (float)(sc * sx);
-        }
-        if (a.gposd) {   // far field (one distance): q is the position
-          a.gposd[2 * q] = sc * sy;
-          a.gposd[2 * q + 1] = sc * sx;
-        }
-        if (a.gnf) {
-          const double nf = a.nf[q % a.nd];
-          a.gnf[q] = (float)(pi * sn / (nf * nf * NN));
-        }
-      }
+    for (int e = 0; e < 3; ++e) v[e] += pp[e];
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int e = 0; e < 3; ++e) v[e] += __shfl_xor_sync(0xffffffffu, v[e], o);
+  if ((threadIdx.x & 31) == 0)
+    for (int e = 0; e < 3; ++e) red[3 * (threadIdx.x >> 5) + e] = v[e];
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 4; ++w)
+      for (int e = 0; e < 3; ++e) v[e] += red[3 * w + e];
+    const double pi = 3.14159265358979323846, NN = (double)a.N * a.N, sc = 2.0 * pi / NN;
+    if (a.gpos) {
+      a.gpos[2 * q] = (float)(sc * v[0]);
+      a.gpos[2 * q + 1] = (float)(sc * v[1]);
+    }
+    if (a.gposd) {   // far field (one distance): q is the position
+      a.gposd[2 * q] = sc * v[0];
+      a.gposd[2 * q + 1] = sc * v[1];
+    }
+    if (a.gnf) {
+      const double nf = a.nf[q % a.nd];
+      a.gnf[q] = (float)(pi * v[2] / (nf * nf * NN));
     }
   }
 }
@@ -886,13 +914,47 @@ __global__ void k_add2(float2* __restrict__ g, const float2* __restrict__ q, siz
 }
 
 // ============================================================================ launch sequence
+// The stream a sequence of row and column kernels goes to.  `chained`: the work enqueued last is one of
+// them, so that the next may overlap its prologue with it; the first of a run, or the first after other
+// work or an event wait, is launched in plain stream order (everything earlier has completed by then,
+// the tables, the transmission and the status word among it).  With the warp-local rows, the twiddle
+// tables by stage and the early transmission loads: 64 x 8 far field at N = 256 1243 -> 1143 us, 8 x 4
+// holograms of 1024 798 -> 761 us.
+// Not while a graph is captured: graphs with programmatic edges were instantiated anew for each request
+// of a served shape instead of updated (burst of 12 requests 3.57 -> 4.55 ms).
+struct Seq {
+  cudaStream_t s;
+  bool overlap = false, chained = false;
+  cudaError_t err = cudaSuccess;
+  explicit Seq(cudaStream_t stream) : s(stream) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    overlap = cudaStreamIsCapturing(stream, &st) == cudaSuccess && st == cudaStreamCaptureStatusNone;
+  }
+  void launch(void (*kernel)(TPArgs), dim3 grid, int smem, const TPArgs& a) {
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = dim3(NT2);
+    c.dynamicSmemBytes = (size_t)smem;
+    c.stream = s;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &at;
+    c.numAttrs = overlap && chained ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&c, kernel, a);
+    if (e != cudaSuccess && err == cudaSuccess) err = e;
+    note_launch();
+    chained = true;
+  }
+};
+
 template <int N, int MODE>
-static void row(const TPArgs& a, int gy, cudaStream_t s) {
-  (k_row<N, MODE><<<dim3(N / Geo2<N>::RB, gy), NT2, row_smem_bytes<N>(), s>>>(a), note_launch());
+static void row(const TPArgs& a, int gy, Seq& q) {
+  q.launch(k_row<N, MODE>, dim3(N / Geo2<N>::RB, gy), row_smem_bytes<N>(), a);
 }
 template <int N, int MODE>
-static void col(const TPArgs& a, int gy, cudaStream_t s) {
-  (k_col<N, MODE><<<dim3(N / Geo2<N>::CW, gy), NT2, col_smem_bytes<N>(), s>>>(a), note_launch());
+static void col(const TPArgs& a, int gy, Seq& q) {
+  q.launch(k_col<N, MODE>, dim3(N / Geo2<N>::CW, gy), col_smem_bytes<N>(), a);
 }
 
 template <int N, class F>
@@ -914,6 +976,10 @@ static cudaError_t prepare_t2() {
   return e;
 }
 
+
+int twopass_columns(int N) {
+  return N == 256 ? 256 / Geo2<256>::CW : N == 512 ? 512 / Geo2<512>::CW : 1024 / Geo2<1024>::CW;
+}
 
 cudaError_t prepare_twopass(int N) {
   // idempotent; called by every entry point before it enqueues (never inside a stream capture)
@@ -1003,39 +1069,41 @@ static cudaError_t twopass_t(TPArgs a, cudaStream_t s, cudaEvent_t ev0, cudaEven
   // the detector passes (and the separate loss pass) are the first readers of the measured
   // intensities: wait for their copy there, not before the forward passes
   cudaError_t werr = cudaSuccess;
+  Seq q(s);
   auto wait_meas = [&]() {
     if (!meas_ready) return;
     const cudaError_t e = cudaStreamWaitEvent(s, meas_ready, 0);
     if (e != cudaSuccess && werr == cudaSuccess) werr = e;
     meas_ready = nullptr;
+    q.chained = false;
   };
   if (ev0) cudaEventRecord(ev0, s);
   if (far) {
-    row<N, R_PHAT>(a, M, s);
-    col<N, C_PHAT>(a, M, s);
+    row<N, R_PHAT>(a, M, q);
+    col<N, C_PHAT>(a, M, q);
   }
   // ---------------- forward
   for (int m = 0; m < M; ++m) {
     a.m = m;
-    if (far) col<N, C_PSI0>(a, B, s);
+    if (far) col<N, C_PSI0>(a, B, q);
     for (int j = 0; j < L; ++j) {
       a.j = j;
-      row<N, R_FWD>(a, B, s);
+      row<N, R_FWD>(a, B, q);
       if (j < L - 1) {
         a.buf = 0;
         const int jn = j + 1;
         if (jn % a.cp == 0) out_slot(spck, a.ncp, jn / a.cp);
         else if (jn > j0_last) out_slot(spsg, a.cp, jn - j0_last);
         else out_slot(nullptr, 1, 0);
-        col<N, C_PROP>(a, B, s);
+        col<N, C_PROP>(a, B, q);
         a.spec_out = nullptr;
       } else if (far) {
         wait_meas();
-        if (fuse && a.loss == 1) col<N, C_FAR_SEED_P>(a, B, s);
-        else if (fuse) col<N, C_FAR_SEED>(a, B, s);
-        else col<N, C_FAR>(a, B, s);
+        if (fuse && a.loss == 1) col<N, C_FAR_SEED_P>(a, B, q);
+        else if (fuse) col<N, C_FAR_SEED>(a, B, q);
+        else col<N, C_FAR>(a, B, q);
       } else {
-        col<N, C_NEAR_PHI>(a, B, s);
+        col<N, C_NEAR_PHI>(a, B, q);
         const bool parts = meas_ready && meas_part && n_meas_part == a.nd;
         if (!parts) wait_meas();
         for (int d = 0; d < a.nd; ++d) {
@@ -1043,30 +1111,34 @@ static cudaError_t twopass_t(TPArgs a, cudaStream_t s, cudaEvent_t ev0, cudaEven
           if (parts) {   // this distance's intensities only; the later ones are still arriving
             const cudaError_t e = cudaStreamWaitEvent(s, meas_part[d], 0);
             if (e != cudaSuccess && werr == cudaSuccess) werr = e;
+            q.chained = false;
           }
-          if (fuse && a.loss == 1) row<N, R_NEAR_DSEED_P>(a, B, s);
-          else if (fuse) row<N, R_NEAR_DSEED>(a, B, s);
-          else row<N, R_NEAR_DET>(a, B, s);
+          if (fuse && a.loss == 1) row<N, R_NEAR_DSEED_P>(a, B, q);
+          else if (fuse) row<N, R_NEAR_DSEED>(a, B, q);
+          else row<N, R_NEAR_DET>(a, B, q);
         }
       }
     }
   }
   wait_meas();   // (no-op when a detector pass already waited)
-  if (!fuse) (k_loss2<<<dim3((unsigned)(NN / LOSS_PX), B * a.nd), 256, 0, s>>>(a), note_launch());
+  if (!fuse) {
+    (k_loss2<<<dim3((unsigned)(NN / LOSS_PX), B * a.nd), 256, 0, s>>>(a), note_launch());
+    q.chained = false;
+  }
   if (a.adj) {
     // ---------------- adjoint
     for (int m = 0; m < M; ++m) {
       a.m = m;
       if (far) {
-        if (!fuse) col<N, C_SEED>(a, B, s);
+        if (!fuse) col<N, C_SEED>(a, B, q);
       } else {
         if (!fuse) {
           for (int d = 0; d < a.nd; ++d) {
             a.d = d;
-            row<N, R_NEAR_SEED>(a, B, s);
+            row<N, R_NEAR_SEED>(a, B, q);
           }
         }
-        col<N, C_NEAR_Q>(a, B, s);
+        col<N, C_NEAR_Q>(a, B, q);
       }
       for (int sg = a.ncp - 1; sg >= 0; --sg) {
         const int j0 = sg * a.cp, j1 = min(j0 + a.cp, L) - 1;
@@ -1075,20 +1147,20 @@ static cudaError_t twopass_t(TPArgs a, cudaStream_t s, cudaEvent_t ev0, cudaEven
         a.j1 = j1;
         if (sg != a.ncp - 1 && j1 > j0) {
           a.j = j0;
-          row<N, R_RC_FIRST>(a, B, s);
+          row<N, R_RC_FIRST>(a, B, q);
           for (int j = j0 + 1; j <= j1; ++j) {
             a.buf = 1;
             a.j = j - 1;                                  // gap j-1 -> j
             out_slot(spsg, a.cp, j - j0);
-            col<N, C_PROP>(a, B, s);
+            col<N, C_PROP>(a, B, q);
             a.spec_out = nullptr;
             a.j = j;
-            row<N, R_RC>(a, B, s);
+            row<N, R_RC>(a, B, q);
           }
         }
         for (int j = j1; j >= j0; --j) {
           a.j = j;
-          row<N, R_ADJ>(a, B, s);
+          row<N, R_ADJ>(a, B, q);
           if (j > 0) {
             a.buf = 0;
             if (want_gap) {
@@ -1096,33 +1168,35 @@ static cudaError_t twopass_t(TPArgs a, cudaStream_t s, cudaEvent_t ev0, cudaEven
               a.spi_n = (j == j0) ? a.ncp : a.cp;
               a.spi_slot = (j == j0) ? sg : j - j0;
             }
-            col<N, C_PROP_ADJ>(a, B, s);
+            col<N, C_PROP_ADJ>(a, B, q);
             a.spec_in = nullptr;
           } else if (far) {
-            col<N, C_Q>(a, B, s);
+            col<N, C_Q>(a, B, q);
           }
         }
       }
     }
   }
   if (ev1) cudaEventRecord(ev1, s);
+  q.chained = false;
   if (a.adj) {
-    (k_final2<<<1, 1024, 0, s>>>(a, nloss, ncol), note_launch());
+    const bool grads = a.posp && (a.gpos || a.gposd || a.gnf);
+    (k_final2<<<1 + (grads ? B * a.nd : 0), 128, 0, s>>>(a, nloss, ncol), note_launch());
     if (want_gap && a.ggap) launch_gap_final(a.gapp, B, L - 1, ncol, a.ggap, s);
     if (a.g_probe) {
       const size_t MNN = (size_t)M * NN;
       // per-element FP64 sum over the batch (deterministic), then back to real space
       launch_qsum(a.qacc, a.qsum, B, MNN, s);
       if (far) {
-        col<N, C_PG>(a, M, s);
-        row<N, R_PG_OUT>(a, M, s);
+        col<N, C_PG>(a, M, q);
+        row<N, R_PG_OUT>(a, M, q);
       } else {
         (k_add2<<<1024, 256, 0, s>>>(a.g_probe, a.qsum, MNN), note_launch());
       }
     }
   }
   const cudaError_t e = cudaGetLastError();
-  return e != cudaSuccess ? e : werr;
+  return e != cudaSuccess ? e : q.err != cudaSuccess ? q.err : werr;
 }
 
 cudaError_t launch_twopass(TPArgs a, cudaStream_t s, cudaEvent_t ev0, cudaEvent_t ev1, cudaEvent_t meas_ready,

@@ -215,6 +215,7 @@ cudaError_t launch_twopass(TPArgs a, cudaStream_t s, cudaEvent_t ev_start, cudaE
                            cudaEvent_t meas_ready = nullptr, const cudaEvent_t* meas_part = nullptr,
                            int n_meas_part = 0);
 cudaError_t prepare_twopass(int N);
+int twopass_columns(int N);   // column CTAs per field: partials per position of the column passes
 // set the dynamic shared-memory attributes of every kernel used for tile size N (call outside capture)
 cudaError_t prepare_path(int N, int farfield);
 
