@@ -284,7 +284,11 @@ int get_tables(adorym_ctx* ctx, const adorym_problem& p, Tables* out) {
   return ADORYM_OK;
 }
 
-int enqueue(const Plan& pl, const Object& obj, const Tables& tab, const CallPtrs& c, char* ws, cudaStream_t s,
+// Boxes from which the probe kernels run on the side stream.  Below, the box kernels are shorter than two
+// forks and joins, and the call is one chain.
+constexpr size_t kSideVoxels = (size_t)1 << 17;
+
+int enqueue(const Plan& pl, const Object& obj, const Tables& tab, const CallPtrs& c, char* ws, cudaStream_t stream,
             std::string* err, cudaEvent_t ev_start, cudaEvent_t ev_stop) {
   const adorym_problem& p = pl.p;
   auto W = [&](size_t off) { return ws + off; };
@@ -301,19 +305,20 @@ int enqueue(const Plan& pl, const Object& obj, const Tables& tab, const CallPtrs
   int* box = reinterpret_cast<int*>(W(pl.off_box));
   int* status = c.status ? c.status : reinterpret_cast<int*>(W(pl.off_status));
   bool join_side = false;   // the call's stream waits for the side stream's last kernels
-  if (!c.status && (rc = chk(cudaMemsetAsync(status, 0, sizeof(int), s), "status"))) return rc;
+  Chain s(stream), s2(c.side ? c.side : stream);
   float2* phat = reinterpret_cast<float2*>(W(pl.off_phat));
   // the probe transform needs only the probe: on the side stream it overlaps the passes below
-  const bool side = c.side && !two_pass(p.N);
+    // (only beside box kernels that take longer than the forks and joins)
+  const bool side = c.side && !two_pass(p.N) && V >= kSideVoxels;
   if (side && pl.far) {
-    if ((rc = chk(cudaEventRecord(c.ev_side[0], s), "fork"))) return rc;
+    if ((rc = chk(cudaEventRecord(c.ev_side[0], stream), "fork"))) return rc;
     if ((rc = chk(cudaStreamWaitEvent(c.side, c.ev_side[0], 0), "fork"))) return rc;
-    if ((rc = chk(launch_probe_hat(p.N, p.M, c.probe, phat, tab.tw(), c.side), "probe_hat"))) return rc;
+    if ((rc = chk(launch_probe_hat(p.N, p.M, c.probe, phat, tab.tw(), s2), "probe_hat"))) return rc;
     if ((rc = chk(cudaEventRecord(c.ev_side[1], c.side), "join"))) return rc;
   }
   int* hctl = pl.helpers ? reinterpret_cast<int*>(W(pl.off_hctl)) : nullptr;
   if ((rc = chk(launch_bbox(c.pos, p.B, p.N, p.Ly, p.Lx, pl.far ? 1 : 0, pl.tomo ? 1 : 0, box, 2 * p.B * pl.nd, status,
-                            s, hctl, (int)helper_ctl_ints(pl)),
+                            !c.status || c.status_clear, s, hctl, (int)helper_ctl_ints(pl)),
                 "bbox")))
     return rc;
   // near field with one probe mode: one term per voxel and call, added in place by the kernels
@@ -333,7 +338,9 @@ int enqueue(const Plan& pl, const Object& obj, const Tables& tab, const CallPtrs
   // above and the probe transform do not read them); the two-pass sequence waits inside, before
   // its detector passes
   auto wait_meas = [&]() -> int {
-    return c.meas_ready ? chk(cudaStreamWaitEvent(s, c.meas_ready, 0), "wait for intensities") : ADORYM_OK;
+    if (!c.meas_ready) return ADORYM_OK;
+    s.breaks();
+    return chk(cudaStreamWaitEvent(stream, c.meas_ready, 0), "wait for intensities");
   };
   if (two_pass(p.N)) {
     TPArgs t{};
@@ -400,7 +407,8 @@ int enqueue(const Plan& pl, const Object& obj, const Tables& tab, const CallPtrs
       return rc;
   } else {
     if (pl.far) {
-      rc = side ? chk(cudaStreamWaitEvent(s, c.ev_side[1], 0), "join")
+      if (side) s.breaks();
+      rc = side ? chk(cudaStreamWaitEvent(stream, c.ev_side[1], 0), "join")
                 : chk(launch_probe_hat(p.N, p.M, c.probe, phat, tab.tw(), s), "probe_hat");
       if (rc) return rc;
     }
@@ -465,17 +473,25 @@ int enqueue(const Plan& pl, const Object& obj, const Tables& tab, const CallPtrs
     a.gI = reinterpret_cast<float*>(W(pl.off_gI));
     a.lossp = reinterpret_cast<double*>(W(pl.off_lossp));
     if ((rc = wait_meas())) return rc;
-    if (ev_start) cudaEventRecord(ev_start, s);
+    if (ev_start) {
+      cudaEventRecord(ev_start, stream);
+      s.breaks();
+    }
     if ((rc = chk(launch_path(a, pl.far ? 1 : 0, s), "path"))) return rc;
-    if (ev_stop) cudaEventRecord(ev_stop, s);
+    if (ev_stop) {
+      cudaEventRecord(ev_stop, stream);
+      s.breaks();
+    }
     if (pl.want_gaps && c.g_gaps) {
       if ((rc = chk(launch_gap_final(a.gapp, p.B, p.L - 1, 1, c.g_gaps, s), "gap_final"))) return rc;
     }
     if (pl.adj && (pl.want_probe || c.loss)) {
       // the probe-gradient kernels (one CTA per mode) run beside the object-gradient pass
-      cudaStream_t sp = side ? c.side : s;
+      Chain& sp = side ? s2 : s;
       if (side) {
-        if ((rc = chk(cudaEventRecord(c.ev_side[2], s), "fork"))) return rc;
+        s2.breaks();
+        if ((rc = chk(cudaEventRecord(c.ev_side[2], stream), "fork"))) return rc;
+        s.breaks();
         if ((rc = chk(cudaStreamWaitEvent(c.side, c.ev_side[2], 0), "fork"))) return rc;
       }
       if ((rc = chk(launch_probe_grad(p.N, p.M, p.B, pl.far ? 1 : 0, a.qacc, reinterpret_cast<float2*>(W(pl.off_qsum)),
@@ -501,7 +517,7 @@ int enqueue(const Plan& pl, const Object& obj, const Tables& tab, const CallPtrs
       rc = chk(launch_grad_add(gd, gb, c.gd, c.gb, p.Lz, p.Ly, p.Lx, box, s), "grad_add");
     if (rc) return rc;
   }
-  if (join_side && (rc = chk(cudaStreamWaitEvent(s, c.ev_side[3], 0), "join"))) return rc;
+  if (join_side && (rc = chk(cudaStreamWaitEvent(stream, c.ev_side[3], 0), "join"))) return rc;
   return ADORYM_OK;
 }
 
@@ -790,6 +806,21 @@ static int run_call(adorym_ctx* ctx, const adorym_problem* p, int obj_id, const 
   }
   if (g_pos) c.g_pos = host_gpos ? reinterpret_cast<float*>(ws + pl.off_s_gpos) : g_pos;
   if (I_out) c.I_out = host_iout ? reinterpret_cast<float*>(ws + pl.off_s_iout) : I_out;
+  // the call's status word is a mapped host int, written by the call's first kernel and again only by one that
+  // finds an error (read by adorym_check, or below)
+  if (!ctx->status_host) {
+    void *h = nullptr, *d = nullptr;
+    if (cudaHostAlloc(&h, sizeof(int), cudaHostAllocMapped) != cudaSuccess ||
+        cudaHostGetDevicePointer(&d, h, 0) != cudaSuccess) {
+      if (h) cudaFreeHost(h);
+      return cuda_fail(ctx, cudaGetLastError(), "status");
+    }
+    ctx->status_host = static_cast<int*>(h);
+    ctx->status_dev = static_cast<int*>(d);
+    *ctx->status_host = 0;
+  }
+  c.status = ctx->status_dev;
+  c.status_clear = true;
   if (ctx->timing && !ctx->ev0) {
     cudaEventCreate(&ctx->ev0);
     cudaEventCreate(&ctx->ev1);
@@ -839,13 +870,6 @@ static int run_call(adorym_ctx* ctx, const adorym_problem* p, int obj_id, const 
     cudaMemcpyAsync(g_offset, c.g_offset, 2 * sizeof(float), cudaMemcpyDeviceToHost, s);
     sync_after = true;
   }
-  // the call's status word goes to a pinned host int (read by adorym_check, or below)
-  if (!ctx->status_host) {
-    void* h = nullptr;
-    if (cudaHostAlloc(&h, sizeof(int), cudaHostAllocDefault) != cudaSuccess) return cuda_fail(ctx, cudaGetLastError(), "status");
-    ctx->status_host = static_cast<int*>(h);
-  }
-  cudaMemcpyAsync(ctx->status_host, ws + pl.off_status, sizeof(int), cudaMemcpyDeviceToHost, s);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(ctx, e, "enqueue");
   if (sync_after) {

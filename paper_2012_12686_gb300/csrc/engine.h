@@ -80,9 +80,10 @@ struct CallPtrs {
   // transform beside the object-gradient pass.  Null: everything on the call's stream.
   cudaStream_t side = nullptr;
   cudaEvent_t ev_side[4] = {nullptr, nullptr, nullptr, nullptr};
-  // device-visible status word to use instead of the plan's (not cleared by the call: the owner
-  // zeroes it before the work runs); null: the workspace word, cleared on the stream
+  // device-visible status word to use instead of the plan's, cleared by the call's first kernel with
+  // status_clear, else by its owner before the work runs; null: the workspace word, cleared
   int* status = nullptr;
+  bool status_clear = false;
 };
 
 int validate(const adorym_problem& p, const char** err);
@@ -131,7 +132,8 @@ struct adorym_ctx {
   cudaStream_t copy_stream = nullptr;          // host-to-device copy of measured intensities
   cudaEvent_t ev_fork = nullptr, ev_meas = nullptr;
   cudaEvent_t ev_meas_d[4] = {nullptr, nullptr, nullptr, nullptr};   // per-distance intensity copies
-  int* status_host = nullptr;                  // pinned copy of the last call's status word
+  int* status_host = nullptr;                  // mapped host word: the last call's status
+  int* status_dev = nullptr;                   // the same word as the device sees it
   cudaStream_t side_stream = nullptr;          // single-CTA probe kernels (CallPtrs::side)
   cudaEvent_t ev_side[4] = {nullptr, nullptr, nullptr, nullptr};
   int inject_alloc_failures = 0;               // adorym_inject_alloc_failures: pending count

@@ -22,7 +22,9 @@ __global__ void __launch_bounds__(Geo<N>::NT) k_probe_hat(const float2* __restri
   extern __shared__ float2 sm[];
   float2* A = sm;
   float2* tw = A + X::FIELD;
+  allow_next();
   X::fill_twiddles(tw, twg);
+  after_previous();
   const float2* p = probe + (size_t)blockIdx.x * N * N;
   float2* o = phat + (size_t)blockIdx.x * N * N;
   using V1 = float2[CY];
@@ -48,8 +50,10 @@ __global__ void __launch_bounds__(Geo<N>::NT) k_probe_hat(const float2* __restri
 // Block of 256 threads = 32 consecutive elements x 8 batch chunks; each thread sums its chunk
 // Kahan-compensated in FP32 (loads issued four at a time), then the 8 partials of an element are
 // added in FP64 in chunk order (deterministic).
-__global__ void __launch_bounds__(256) k_qsum(const float2* __restrict__ qacc, float2* __restrict__ qsum, int B,
+__global__ void __launch_bounds__(256) k_qsum(const float2* qacc, float2* __restrict__ qsum, int B,
                                               size_t MNN) {
+  allow_next();
+  after_previous();
   __shared__ double2 part[8][32];
   const int e = threadIdx.x & 31, c = threadIdx.x >> 5;
   const size_t i = (size_t)blockIdx.x * 32 + e;
@@ -58,7 +62,7 @@ __global__ void __launch_bounds__(256) k_qsum(const float2* __restrict__ qacc, f
   if (i < MNN) {
 #pragma unroll 4
     for (int b = b0; b < b1; ++b) {
-      const float2 v = __ldg(qacc + (size_t)b * MNN + i);
+      const float2 v = __ldcg(qacc + (size_t)b * MNN + i);
       sr.add(v.x);
       si.add(v.y);
     }
@@ -77,14 +81,16 @@ __global__ void __launch_bounds__(256) k_qsum(const float2* __restrict__ qacc, f
 }
 
 // The same for a batch too small to split: a thread per element, the batch in its own order.
-__global__ void __launch_bounds__(256) k_qsum_few(const float2* __restrict__ qacc, float2* __restrict__ qsum, int B,
+__global__ void __launch_bounds__(256) k_qsum_few(const float2* qacc, float2* __restrict__ qsum, int B,
                                                   size_t MNN) {
+  allow_next();
+  after_previous();
   const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
   if (i >= MNN) return;
   Kahan sr, si;
 #pragma unroll 4
   for (int b = 0; b < B; ++b) {
-    const float2 v = __ldg(qacc + (size_t)b * MNN + i);
+    const float2 v = __ldcg(qacc + (size_t)b * MNN + i);
     sr.add(v.x);
     si.add(v.y);
   }
@@ -94,14 +100,16 @@ __global__ void __launch_bounds__(256) k_qsum_few(const float2* __restrict__ qac
 // g_gap[j] = sum of gap j's partials over the positions and column CTAs, one CTA per gap, threads strided
 // over the partials, then a fixed tree.  (Gaps walked by the threads of one CTA, one after the other over
 // the batch, took 40 us for 7 gaps and 100 positions.)
-__global__ void __launch_bounds__(128) k_gap_final(const double* __restrict__ gapp, int B, int ngap, int parts,
+__global__ void __launch_bounds__(128) k_gap_final(const double* gapp, int B, int ngap, int parts,
                                                    float* __restrict__ g) {
   __shared__ double red[4];
+  allow_next();
+  after_previous();
   const int j = blockIdx.x;
   double s = 0.0;
 #pragma unroll 4
   for (int i = threadIdx.x; i < B * parts; i += 128)
-    s += gapp[((size_t)(i / parts) * ngap + j) * parts + i % parts];
+    s += __ldcg(gapp + ((size_t)(i / parts) * ngap + j) * parts + i % parts);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
@@ -112,11 +120,13 @@ __global__ void __launch_bounds__(128) k_gap_final(const double* __restrict__ ga
 // Per-angle position offset of ptychotomography (Sec. 2.3.2): one correction vector shifts every
 // position of an angle, so its gradient is the sum of that batch's position gradients.  One warp:
 // lane l adds positions l, l + 32, ... in FP64, then a fixed shuffle tree (deterministic).
-__global__ void k_offset_sum(const double* __restrict__ gposd, int B, float* __restrict__ g_off) {
+__global__ void k_offset_sum(const double* gposd, int B, float* __restrict__ g_off) {
+  allow_next();
+  after_previous();
   double sy = 0.0, sx = 0.0;
   for (int b = threadIdx.x; b < B; b += 32) {
-    sy += gposd[2 * (size_t)b];
-    sx += gposd[2 * (size_t)b + 1];
+    sy += __ldcg(gposd + 2 * (size_t)b);
+    sx += __ldcg(gposd + 2 * (size_t)b + 1);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -129,29 +139,24 @@ __global__ void k_offset_sum(const double* __restrict__ gposd, int B, float* __r
   }
 }
 
-cudaError_t launch_offset_sum(const double* gposd, int B, float* g_off, cudaStream_t s) {
-  (k_offset_sum<<<1, 32, 0, s>>>(gposd, B, g_off), note_launch());
-  return cudaGetLastError();
+cudaError_t launch_offset_sum(const double* gposd, int B, float* g_off, Chain& s) {
+  return s.launch(k_offset_sum, 1, 32, 0, gposd, B, g_off);
 }
 
-cudaError_t launch_gap_final(const double* gapp, int B, int ngap, int parts, float* g_gap, cudaStream_t s) {
-  (k_gap_final<<<ngap, 128, 0, s>>>(gapp, B, ngap, parts, g_gap), note_launch());
-  return cudaGetLastError();
+cudaError_t launch_gap_final(const double* gapp, int B, int ngap, int parts, float* g_gap, Chain& s) {
+  return s.launch(k_gap_final, ngap, 128, 0, gapp, B, ngap, parts, g_gap);
 }
 
-cudaError_t launch_qsum(const float2* qacc, float2* qsum, int B, size_t MNN, cudaStream_t s) {
+cudaError_t launch_qsum(const float2* qacc, float2* qsum, int B, size_t MNN, Chain& s) {
   // up to 8 positions the eight batch chunks of k_qsum hold one value or none (21 us for 2 x 512 x 512)
-  if (B <= 8)
-    (k_qsum_few<<<(unsigned)((MNN + 255) / 256), 256, 0, s>>>(qacc, qsum, B, MNN), note_launch());
-  else
-    (k_qsum<<<(unsigned)((MNN + 31) / 32), 256, 0, s>>>(qacc, qsum, B, MNN), note_launch());
-  return cudaGetLastError();
+  if (B <= 8) return s.launch(k_qsum_few, (unsigned)((MNN + 255) / 256), 256, 0, qacc, qsum, B, MNN);
+  return s.launch(k_qsum, (unsigned)((MNN + 31) / 32), 256, 0, qacc, qsum, B, MNN);
 }
 
 // far field: g_probe[m] += IDFT_-{qsum[m]};  near field: g_probe[m] += qsum[m]
 template <int N, int FAR>
-__global__ void __launch_bounds__(Geo<N>::NT) k_probe_grad(const float2* __restrict__ qsum, float2* __restrict__ g,
-                                                         const float2* __restrict__ twg, const double* __restrict__ lossp,
+__global__ void __launch_bounds__(Geo<N>::NT) k_probe_grad(const float2* qsum, float2* __restrict__ g,
+                                                         const float2* __restrict__ twg, const double* lossp,
                                                          int B, double inv_npix, double* __restrict__ loss_out) {
   using X = PathFFT<N>;
   constexpr int CY = X::CY, YS = X::YS, RX = X::RX, KXS = X::KXS, NT = Geo<N>::NT;
@@ -159,12 +164,15 @@ __global__ void __launch_bounds__(Geo<N>::NT) k_probe_grad(const float2* __restr
   extern __shared__ float2 sm[];
   float2* A = sm;
   float2* tw = A + X::FIELD;
+  allow_next();
+  if (FAR && g) X::fill_twiddles(tw, twg);
+  after_previous();
   if (loss_out && blockIdx.x == 0 && threadIdx.x < 32) {
     // FP64 sum of the per-position partials in a fixed order: lane l adds positions l, l + 32, ...
     // in turn, then a fixed xor tree over the lanes (one warp keeps B / 32 loads in flight instead of
     // one thread walking all B partials)
     double s = 0.0;
-    for (int b = (int)threadIdx.x; b < B; b += 32) s += lossp[b];
+    for (int b = (int)threadIdx.x; b < B; b += 32) s += __ldcg(lossp + b);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (threadIdx.x == 0) *loss_out = s * inv_npix;
@@ -173,17 +181,16 @@ __global__ void __launch_bounds__(Geo<N>::NT) k_probe_grad(const float2* __restr
   const float2* q = qsum + blockIdx.x * NN;
   float2* o = g + blockIdx.x * NN;
   if (!FAR) {
-    for (size_t i = threadIdx.x; i < NN; i += NT) o[i] = cadd(o[i], q[i]);
+    for (size_t i = threadIdx.x; i < NN; i += NT) o[i] = cadd(o[i], __ldcg(q + i));
     return;
   }
-  X::fill_twiddles(tw, twg);
   __syncthreads();
   const float invNN = 1.0f / (float)NN;
   using V1 = float2[CY];
   using V2 = float2[RX];
   X::template r23<0, +1>(A, tw, [&](V2& v, int ky, int t) {
 #pragma unroll
-    for (int i = 0; i < RX; ++i) v[i] = cscale(__ldg(q + ky * N + t + KXS * i), invNN);
+    for (int i = 0; i < RX; ++i) v[i] = cscale(__ldcg(q + ky * N + t + KXS * i), invNN);
   });
   X::row_sync();
   X::template inv_pair<+1>(A, tw);
@@ -208,7 +215,7 @@ int path_smem_bytes(int N) {
   }
 }
 
-cudaError_t launch_path(const PathArgs& a, int farfield, cudaStream_t s) {
+cudaError_t launch_path(const PathArgs& a, int farfield, Chain& s) {
   if (a.hyj) return launch_path_gaps(a, farfield, s);   // variable slice spacing
   if (a.pipe) return launch_path_pipe(a, farfield, s);
   if (a.helpers) return launch_path_help(a, farfield, s);
@@ -233,13 +240,12 @@ constexpr int probe_smem_bytes() {   // field + twiddle tables
 }
 
 template <int N>
-static cudaError_t launch_probe_hat_t(int M, const float2* probe, float2* phat, const float2* tw, cudaStream_t s) {
+static cudaError_t launch_probe_hat_t(int M, const float2* probe, float2* phat, const float2* tw, Chain& s) {
   const int smem = probe_smem_bytes<N>();
-  (k_probe_hat<N><<<M, Geo<N>::NT, smem, s>>>(probe, phat, tw), note_launch());
-  return cudaGetLastError();
+  return s.launch(k_probe_hat<N>, M, Geo<N>::NT, smem, probe, phat, tw);
 }
 
-cudaError_t launch_probe_hat(int N, int M, const float2* probe, float2* phat, const float2* tw, cudaStream_t s) {
+cudaError_t launch_probe_hat(int N, int M, const float2* probe, float2* phat, const float2* tw, Chain& s) {
   switch (N) {
     case 8: return launch_probe_hat_t<8>(M, probe, phat, tw, s);
     case 16: return launch_probe_hat_t<16>(M, probe, phat, tw, s);
@@ -252,17 +258,19 @@ cudaError_t launch_probe_hat(int N, int M, const float2* probe, float2* phat, co
 
 template <int N, int FAR>
 static cudaError_t launch_probe_grad_t(int M, int B, const float2* qacc, float2* qsum, float2* g, const float2* tw,
-                                       const double* lossp, double inv_npix, double* loss_out, cudaStream_t s) {
+                                       const double* lossp, double inv_npix, double* loss_out, Chain& s) {
   const size_t MNN = (size_t)M * N * N;
-  if (g) launch_qsum(qacc, qsum, B, MNN, s);
+  if (g) {
+    const cudaError_t e = launch_qsum(qacc, qsum, B, MNN, s);
+    if (e != cudaSuccess) return e;
+  }
   const int smem = probe_smem_bytes<N>();
-  (k_probe_grad<N, FAR><<<M, Geo<N>::NT, smem, s>>>(qsum, g, tw, lossp, B, inv_npix, loss_out), note_launch());
-  return cudaGetLastError();
+  return s.launch(k_probe_grad<N, FAR>, M, Geo<N>::NT, smem, qsum, g, tw, lossp, B, inv_npix, loss_out);
 }
 
 cudaError_t launch_probe_grad(int N, int M, int B, int farfield, const float2* qacc, float2* qsum, float2* g_probe,
                               const float2* tw, const double* lossp, double inv_npix, double* loss_out,
-                              cudaStream_t s) {
+                              Chain& s) {
   switch (N) {
 #define ADORYM_CASE(n)                                                                                     \
   case n:                                                                                                  \

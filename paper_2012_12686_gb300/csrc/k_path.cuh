@@ -142,6 +142,7 @@ __device__ __forceinline__ void path_body(const PathArgs& a) {
   const int b = PIPE ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
   const int rank = PIPE ? (int)(blockIdx.x & 1) : 0;   // cluster of two CTAs along x
   const int M = a.M, L = a.L, cp = a.cp, ncp = a.ncp;
+  allow_next();
   X::fill_twiddles(tw, a.tw);
   for (int i = threadIdx.x; i < N; i += NT) {
     hy[i] = a.hy[i];
@@ -157,6 +158,7 @@ __device__ __forceinline__ void path_body(const PathArgs& a) {
     ramp_table(ry, (float)(py - fy), N, NT);
     ramp_table(rx, (float)(px - fx), N, NT);
   }
+  after_previous();
   __syncthreads();
 
   const int Ly = a.Ly, Lx = a.Lx;
@@ -168,7 +170,7 @@ __device__ __forceinline__ void path_body(const PathArgs& a) {
   const size_t slab = (size_t)Ly * Lx;
   auto tload = [&](int j, int y, int x) -> float2 {
     const int gy = p0y + y, gx = p0x + x, gz = FAR ? j : b * L + j;
-    if (gy >= 0 && gy < Ly && gx >= 0 && gx < Lx) return __ldg(a.T + ((size_t)gz * Ly + gy) * Lx + gx);
+    if (gy >= 0 && gy < Ly && gx >= 0 && gx < Lx) return a.T[((size_t)gz * Ly + gy) * Lx + gx];
     return make_float2(1.f, 0.f);
   };
   // offset of patch pixel (t, x) of slice j in the volume (interior patches)
@@ -179,7 +181,7 @@ __device__ __forceinline__ void path_body(const PathArgs& a) {
     if (interior) {
       const float2* p = a.T + voff(j, t, x);
 #pragma unroll
-      for (int k = 0; k < CY; ++k) pa[k] = __ldg(p + (size_t)(YS * k) * Lx);
+      for (int k = 0; k < CY; ++k) pa[k] = p[(size_t)(YS * k) * Lx];
     } else {
 #pragma unroll
       for (int k = 0; k < CY; ++k) pa[k] = tload(j, YS * k + t, x);
@@ -302,7 +304,7 @@ __device__ __forceinline__ void path_body(const PathArgs& a) {
 #pragma unroll
         for (int i = 0; i < RX; ++i) {
           const int kx = t + KXS * i;
-          v[i] = cmul(cmul(__ldg(&ph[ky * N + kx]), r), rx[kx]);
+          v[i] = cmul(cmul(ph[ky * N + kx], r), rx[kx]);
         }
       });
       X::row_sync();
@@ -653,7 +655,7 @@ __device__ __forceinline__ void path_body(const PathArgs& a) {
           for (int i = 0; i < RX; ++i) {
             const int kx = t + KXS * i, p = ky * N + kx;
             const float2 r = cmul(r_y, rx[kx]);
-            const float2 base = cmul(cconj(v[i]), cmul(__ldg(&ph[p]), r));
+            const float2 base = cmul(cconj(v[i]), cmul(ph[p], r));
             ay += fyk * base.y;
             ax += freqf1(kx, N) * base.y;
             if (q) q[p] = cmulc(v[i], r);
@@ -707,6 +709,7 @@ __device__ __forceinline__ void helper_body(const PathArgs& a) {
   float2* hy = tw + X::TW;
   float2* hx = hy + N;
   __shared__ int h_task;
+  allow_next();
   X::fill_twiddles(tw, a.tw);
   for (int i = threadIdx.x; i < N; i += NT) {
     hy[i] = a.hy[i];
@@ -714,6 +717,7 @@ __device__ __forceinline__ void helper_body(const PathArgs& a) {
   }
   const int M = a.M, L = a.L, cp = a.cp, ncp = a.ncp, B = a.B, Ly = a.Ly, Lx = a.Lx;
   const int MB = M * B, ntask = (ncp - 1) * MB;
+  after_previous();
   for (;;) {
     if (threadIdx.x == 0) {
       int got = -1;
@@ -742,12 +746,12 @@ __device__ __forceinline__ void helper_body(const PathArgs& a) {
       if (interior) {
         const float2* p = a.T + (gz * Ly + (p0y + t)) * Lx + (p0x + x);
 #pragma unroll
-        for (int k = 0; k < CY; ++k) pa[k] = __ldg(p + (size_t)(YS * k) * Lx);
+        for (int k = 0; k < CY; ++k) pa[k] = p[(size_t)(YS * k) * Lx];
       } else {
 #pragma unroll
         for (int k = 0; k < CY; ++k) {
           const int gy = p0y + YS * k + t, gx = p0x + x;
-          pa[k] = (gy >= 0 && gy < Ly && gx >= 0 && gx < Lx) ? __ldg(a.T + (gz * Ly + gy) * Lx + gx)
+          pa[k] = (gy >= 0 && gy < Ly && gx >= 0 && gx < Lx) ? a.T[(gz * Ly + gy) * Lx + gx]
                                                              : make_float2(1.f, 0.f);
         }
       }
@@ -828,22 +832,19 @@ constexpr int path_smem_bytes_t() {
 }
 
 template <int N, int FAR, bool GAP>
-cudaError_t launch_path_t(const PathArgs& a, cudaStream_t s) {
-  (k_path<N, FAR, GAP><<<a.B, Geo<N>::NT, path_smem_bytes_t<N>(), s>>>(a), note_launch());
-  return cudaGetLastError();
+cudaError_t launch_path_t(const PathArgs& a, Chain& s) {
+  return s.launch(k_path<N, FAR, GAP>, a.B, Geo<N>::NT, path_smem_bytes_t<N>(), a);
 }
 
 template <int N, int FAR>
-cudaError_t launch_path_help_t(const PathArgs& a, cudaStream_t s) {
+cudaError_t launch_path_help_t(const PathArgs& a, Chain& s) {
   // positions, then the recompute helpers
-  (k_path_help<N, FAR><<<a.B + a.helpers, Geo<N>::NT, path_smem_bytes_t<N>(), s>>>(a), note_launch());
-  return cudaGetLastError();
+  return s.launch(k_path_help<N, FAR>, a.B + a.helpers, Geo<N>::NT, path_smem_bytes_t<N>(), a);
 }
 
 template <int N, int FAR>
-cudaError_t launch_path_pipe_t(const PathArgs& a, cudaStream_t s) {
-  (k_path_pipe<N, FAR><<<2 * a.B, Geo<N>::NT, path_smem_bytes_t<N>(), s>>>(a), note_launch());
-  return cudaGetLastError();
+cudaError_t launch_path_pipe_t(const PathArgs& a, Chain& s) {
+  return s.launch(k_path_pipe<N, FAR>, 2 * a.B, Geo<N>::NT, path_smem_bytes_t<N>(), a);
 }
 
 template <int N, int FAR, bool GAP>

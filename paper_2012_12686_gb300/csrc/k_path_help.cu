@@ -5,7 +5,7 @@
 
 namespace adorym {
 
-cudaError_t launch_path_help(const PathArgs& a, int farfield, cudaStream_t s) {
+cudaError_t launch_path_help(const PathArgs& a, int farfield, Chain& s) {
   switch (a.N) {
 #define ADORYM_CASE(n)                                                                  \
   case n:                                                                               \

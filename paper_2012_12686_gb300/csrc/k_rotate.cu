@@ -37,8 +37,11 @@ __device__ __forceinline__ Tap tap(int zt, int xt, int Lz, int Lx, float c, floa
 // full_x the column range is the whole width (tomography: the rotation transpose mixes x and z).
 __global__ void __launch_bounds__(256) k_bbox(const float* __restrict__ pos, int B, int N, int Ly, int Lx, int far,
                                               int full_x, int* __restrict__ box, int npos_values,
-                                              int* __restrict__ status, int* __restrict__ zero, int nzero) {
+                                              int* __restrict__ status, int clear, int* __restrict__ zero,
+                                              int nzero) {
   __shared__ int red[4][8];
+  allow_next();
+  after_previous();
   for (int i = threadIdx.x; i < nzero; i += 256) zero[i] = 0;
   // input check: every position / shift value finite and within +-2^24 px
   bool bad = false;
@@ -46,7 +49,11 @@ __global__ void __launch_bounds__(256) k_bbox(const float* __restrict__ pos, int
     const float v = pos[i];
     bad |= !(fabsf(v) <= 16777216.f);   // also catches NaN
   }
-  if (__syncthreads_or(bad) && threadIdx.x == 0) set_status(status, STATUS_BAD_POSITION);
+  const bool any = __syncthreads_or(bad) != 0;
+  if (threadIdx.x == 0) {
+    if (clear) *status = any ? STATUS_BAD_POSITION : 0;   // the first kernel of the call to write the word
+    else if (any) set_status(status, STATUS_BAD_POSITION);
+  }
   int y0 = 1 << 30, y1 = -(1 << 30), x0 = 1 << 30, x1 = -(1 << 30);
   if (far) {
     for (int b = threadIdx.x; b < B; b += 256) {
@@ -97,12 +104,13 @@ struct Region {
   size_t n;   // Lz * h * w
 };
 
-__device__ __forceinline__ Region region(const int* __restrict__ box, int Lz) {
+// (clamped to the volume whatever the words hold: they index it)
+__device__ __forceinline__ Region region(const int* box, int Lz, int Ly, int Lx) {
   Region r;
-  r.y0 = box[0];
-  r.h = max(0, box[1] - box[0]);
-  r.x0 = box[2];
-  r.w = max(0, box[3] - box[2]);
+  r.y0 = min(max(__ldcg(box), 0), Ly);
+  r.h = min(max(__ldcg(box + 1), r.y0), Ly) - r.y0;
+  r.x0 = min(max(__ldcg(box + 2), 0), Lx);
+  r.w = min(max(__ldcg(box + 3), r.x0), Lx) - r.x0;
   r.n = (size_t)Lz * r.h * r.w;
   return r;
 }
@@ -137,9 +145,11 @@ struct BoxChunks {
 template <bool ROT>
 __global__ void __launch_bounds__(256) k_transmission(const float* __restrict__ vd, const float* __restrict__ vb,
                                                       float2* __restrict__ T, int Lz, int Ly, int Lx, float kdz,
-                                                      float c, float s, const int* __restrict__ box,
+                                                      float c, float s, const int* box,
                                                       double* __restrict__ zero_a, double* __restrict__ zero_b) {
-  const Region R = region(box, Lz);
+  allow_next();
+  after_previous();
+  const Region R = region(box, Lz, Ly, Lx);
   BoxChunks K(R, Lz);
   constexpr int U = BoxChunks::PER_LANE;
   for (unsigned item = K.first(); item < K.items; item += K.stride()) {
@@ -212,6 +222,8 @@ __global__ void __launch_bounds__(256) k_transmission(const float* __restrict__ 
 // forward pass's own bilinear weights, in the order z_t, then x_t ascending.  Table planes of
 // P = Lz * Lx ints: [0] count, [1 + k] packed node z_t * 65536 + x_t, [1 + kRotTaps + k] weight.
 __global__ void __launch_bounds__(256) k_rotate_table(int* __restrict__ tab, int Lz, int Lx, float c, float s) {
+  allow_next();
+  after_previous();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int P = Lz * Lx;
   if (i >= P) return;
@@ -252,10 +264,12 @@ __global__ void __launch_bounds__(256) k_rotate_table(int* __restrict__ tab, int
 // the table (flat index over the box's rows and columns, threads along x).  The taps are FP64
 // sums over positions; each is narrowed once (integer arithmetic, round to nearest) and the
 // weighted taps are added in FP32 in the table's order, like the caller's FP32 gradient
-__global__ void __launch_bounds__(256) k_rotate_adj(const double* __restrict__ gdr, const double* __restrict__ gbr,
+__global__ void __launch_bounds__(256) k_rotate_adj(const double* gdr, const double* gbr,
                                                     float* __restrict__ gd, float* __restrict__ gb, int Lz, int Ly,
-                                                    int Lx, const int* __restrict__ tab, const int* __restrict__ box) {
-  const Region R = region(box, Lz);
+                                                    int Lx, const int* tab, const int* box) {
+  allow_next();
+  after_previous();
+  const Region R = region(box, Lz, Ly, Lx);
   const int P = Lz * Lx;
   const unsigned n = (unsigned)R.n;
   for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -263,11 +277,11 @@ __global__ void __launch_bounds__(256) k_rotate_adj(const double* __restrict__ g
     const int x = R.x0 + (int)(i - row * (unsigned)R.w);
     const int z = (int)(row / (unsigned)R.h), y = R.y0 + (int)(row - (unsigned)z * (unsigned)R.h);
     const int node = z * Lx + x;
-    const int cnt = __ldg(tab + node);
+    const int cnt = __ldca(tab + node);
     float ad = 0.f, ab = 0.f;
     for (int k = 0; k < cnt; ++k) {
-      const int zx = __ldg(tab + (size_t)(1 + k) * P + node);
-      const float wk = __int_as_float(__ldg(tab + (size_t)(1 + kRotTaps + k) * P + node));
+      const int zx = __ldca(tab + (size_t)(1 + k) * P + node);
+      const float wk = __int_as_float(__ldca(tab + (size_t)(1 + kRotTaps + k) * P + node));
       const size_t o = ((size_t)(zx >> 16) * Ly + y) * Lx + (zx & 0xFFFF);
       ad = fmaf(wk, f64_to_f32(gdr + o), ad);
       ab = fmaf(wk, f64_to_f32(gbr + o), ab);
@@ -280,10 +294,12 @@ __global__ void __launch_bounds__(256) k_rotate_adj(const double* __restrict__ g
 
 // FP64 object-gradient accumulators (zeroed over the box by the transmission pass): add the box
 // into the caller's gradient (work split as in BoxChunks)
-__global__ void __launch_bounds__(256) k_grad_add(const double* __restrict__ ad, const double* __restrict__ ab,
+__global__ void __launch_bounds__(256) k_grad_add(const double* ad, const double* ab,
                                                   float* __restrict__ gd, float* __restrict__ gb, int Lz, int Ly,
-                                                  int Lx, const int* __restrict__ box) {
-  const Region R = region(box, Lz);
+                                                  int Lx, const int* box) {
+  allow_next();
+  after_previous();
+  const Region R = region(box, Lz, Ly, Lx);
   BoxChunks K(R, Lz);
   constexpr int U = BoxChunks::PER_LANE;
   for (unsigned item = K.first(); item < K.items; item += K.stride()) {
@@ -321,34 +337,29 @@ static unsigned box_grid(int Lz, int Ly, int Lx) {
 }
 
 cudaError_t launch_bbox(const float* pos, int B, int N, int Ly, int Lx, int far, int full_x, int* box,
-                        int npos_values, int* status, cudaStream_t s, int* zero, int nzero) {
-  (k_bbox<<<1, 256, 0, s>>>(pos, B, N, Ly, Lx, far, full_x, box, npos_values, status, zero, nzero), note_launch());
-  return cudaGetLastError();
+                        int npos_values, int* status, bool clear, Chain& s, int* zero, int nzero) {
+  return s.launch(k_bbox, 1, 256, 0, pos, B, N, Ly, Lx, far, full_x, box, npos_values, status, clear ? 1 : 0, zero, nzero);
 }
 
 cudaError_t launch_transmission(const float* vd, const float* vb, float2* T, int Lz, int Ly, int Lx, float kdz,
                                 int rotate, float c, float sn, const int* box, double* zero_a, double* zero_b,
-                                cudaStream_t s) {
+                                Chain& s) {
   const unsigned grid = box_grid(Lz, Ly, Lx);
-  if (rotate) (k_transmission<true><<<grid, 256, 0, s>>>(vd, vb, T, Lz, Ly, Lx, kdz, c, sn, box, zero_a, zero_b), note_launch());
-  else (k_transmission<false><<<grid, 256, 0, s>>>(vd, vb, T, Lz, Ly, Lx, kdz, c, sn, box, zero_a, zero_b), note_launch());
-  return cudaGetLastError();
+  return s.launch(rotate ? k_transmission<true> : k_transmission<false>, grid, 256, 0, vd, vb, T, Lz, Ly, Lx, kdz, c, sn,
+                  box, zero_a, zero_b);
 }
 
 cudaError_t launch_rotate_adj(const double* gdr, const double* gbr, float* gd, float* gb, int Lz, int Ly, int Lx,
-                              float c, float sn, const int* box, int* tab, cudaStream_t s) {
+                              float c, float sn, const int* box, int* tab, Chain& s) {
   const int nodes = Lz * Lx;
-  (k_rotate_table<<<(nodes + 255) / 256, 256, 0, s>>>(tab, Lz, Lx, c, sn), note_launch());
-  (k_rotate_adj<<<vol_grid((size_t)Lz * Ly * Lx), 256, 0, s>>>(gdr, gbr, gd, gb, Lz, Ly, Lx, tab, box), note_launch());
-  return cudaGetLastError();
+  const cudaError_t e = s.launch(k_rotate_table, (nodes + 255) / 256, 256, 0, tab, Lz, Lx, c, sn);
+  if (e != cudaSuccess) return e;
+  return s.launch(k_rotate_adj, vol_grid((size_t)Lz * Ly * Lx), 256, 0, gdr, gbr, gd, gb, Lz, Ly, Lx, tab, box);
 }
 
 cudaError_t launch_grad_add(const double* ad, const double* ab, float* gd, float* gb, int Lz, int Ly, int Lx,
-                            const int* box, cudaStream_t s) {
-  (k_grad_add<<<box_grid(Lz, Ly, Lx), 256, 0, s>>>(ad, ab, gd, gb, Lz, Ly, Lx, box), note_launch());
-  return cudaGetLastError();
+                            const int* box, Chain& s) {
+  return s.launch(k_grad_add, box_grid(Lz, Ly, Lx), 256, 0, ad, ab, gd, gb, Lz, Ly, Lx, box);
 }
-
-cudaError_t launch_zero(void* p, size_t bytes, cudaStream_t s) { return cudaMemsetAsync(p, 0, bytes, s); }
 
 }  // namespace adorym

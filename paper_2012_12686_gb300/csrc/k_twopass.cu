@@ -16,7 +16,7 @@
 // keeps both the strided and the contiguous stage accesses free of bank conflicts with the
 // lane index on the x digit, so every global access is coalesced; a warp has its rows through all three
 // stages, so a row kernel has no CTA barrier after its tables.  The kernels of a sequence are chained by
-// programmatic dependent launch (Seq).  The column tile is brought in
+// programmatic dependent launch (Chain).  The column tile is brought in
 // by TMA (a 2-D tensor map over the field buffer, completion on an mbarrier) and lands in the
 // [row][column] layout the first in-place stage reads.  With one probe mode and measured data the
 // detector pass also forms the loss term and the adjoint seed.  Loss and position-gradient
@@ -215,15 +215,6 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, i
       : "memory");
 }
 
-// Programmatic dependent launch: the next kernel of the sequence may start its CTAs as soon as all of
-// this one's have started, and runs its prologue (tables, transmission; nothing the sequence writes)
-// until `after_previous`, which returns once the kernel before it has completed and its writes are
-// visible.  Every CTA calls both, so a kernel that has completed implies all before it.  What the
-// sequence itself writes is read with __ldcg (L2): not invariant to the compiler, and never from an L1
-// line that an earlier kernel of the chain left behind.
-__device__ __forceinline__ void allow_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 // ============================================================================ row kernel
 template <int N, int MODE>
 __global__ void __launch_bounds__(NT2, row_minb<N, MODE>()) k_row(const TPArgs a) {
@@ -333,7 +324,7 @@ __global__ void __launch_bounds__(NT2, row_minb<N, MODE>()) k_row(const TPArgs a
 #pragma unroll
       for (int c = 0; c < CH; ++c) {
         const int k = k0 + c;
-        Tv[h][c] = inside(k) ? __ldg(a.T + orow + N2 * k) : make_float2(1.f, 0.f);
+        Tv[h][c] = inside(k) ? __ldcg(a.T + orow + N2 * k) : make_float2(1.f, 0.f);
         if (ADJ) {
           pv[h][ADJ ? c : 0] = __ldcg(psrc + (size_t)y * N + N2 * k + t);
           if (a.gdf) {
@@ -845,6 +836,8 @@ constexpr int LOSS_PX = 1024;   // pixels per loss CTA (256 threads x 4)
 
 __global__ void __launch_bounds__(256) k_loss2(const TPArgs a) {
   __shared__ double red[8];
+  allow_next();
+  after_previous();
   const size_t NN = (size_t)a.N * a.N;
   const size_t base = (size_t)blockIdx.y * NN;
   Kahan acc;
@@ -866,6 +859,8 @@ __global__ void __launch_bounds__(256) k_loss2(const TPArgs a) {
 // FP64 values a clock, so all of it in one CTA of 32 warps took 20 us (holography) to 35 us (128 positions).
 __global__ void __launch_bounds__(128) k_final2(const TPArgs a, int nloss, int ncolblk) {
   __shared__ double red[12];
+  allow_next();
+  after_previous();
   if (blockIdx.x == 0) {
     if (!a.loss_out) return;
     double acc = 0.0;
@@ -908,53 +903,24 @@ __global__ void __launch_bounds__(128) k_final2(const TPArgs a, int nloss, int n
   }
 }
 
-__global__ void k_add2(float2* __restrict__ g, const float2* __restrict__ q, size_t n) {
+__global__ void k_add2(float2* __restrict__ g, const float2* q, size_t n) {
+  allow_next();
+  after_previous();
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-    g[i] = cadd(g[i], q[i]);
+    g[i] = cadd(g[i], __ldcg(q + i));
 }
 
 // ============================================================================ launch sequence
-// The stream a sequence of row and column kernels goes to.  `chained`: the work enqueued last is one of
-// them, so that the next may overlap its prologue with it; the first of a run, or the first after other
-// work or an event wait, is launched in plain stream order (everything earlier has completed by then,
-// the tables, the transmission and the status word among it).  With the warp-local rows, the twiddle
-// tables by stage and the early transmission loads: 64 x 8 far field at N = 256 1243 -> 1143 us, 8 x 4
-// holograms of 1024 798 -> 761 us.
-// Not while a graph is captured: graphs with programmatic edges were instantiated anew for each request
-// of a served shape instead of updated (burst of 12 requests 3.57 -> 4.55 ms).
-struct Seq {
-  cudaStream_t s;
-  bool overlap = false, chained = false;
-  cudaError_t err = cudaSuccess;
-  explicit Seq(cudaStream_t stream) : s(stream) {
-    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    overlap = cudaStreamIsCapturing(stream, &st) == cudaSuccess && st == cudaStreamCaptureStatusNone;
-  }
-  void launch(void (*kernel)(TPArgs), dim3 grid, int smem, const TPArgs& a) {
-    cudaLaunchConfig_t c{};
-    c.gridDim = grid;
-    c.blockDim = dim3(NT2);
-    c.dynamicSmemBytes = (size_t)smem;
-    c.stream = s;
-    cudaLaunchAttribute at;
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    c.attrs = &at;
-    c.numAttrs = overlap && chained ? 1 : 0;
-    const cudaError_t e = cudaLaunchKernelEx(&c, kernel, a);
-    if (e != cudaSuccess && err == cudaSuccess) err = e;
-    note_launch();
-    chained = true;
-  }
-};
-
+// Row and column kernels of a Chain: tables are filled while the kernel before drains.  With the warp-local
+// rows, the twiddle tables by stage and the early transmission loads: 64 x 8 far field at N = 256 1243 ->
+// 1143 us, 8 x 4 holograms of 1024 798 -> 761 us.
 template <int N, int MODE>
-static void row(const TPArgs& a, int gy, Seq& q) {
-  q.launch(k_row<N, MODE>, dim3(N / Geo2<N>::RB, gy), row_smem_bytes<N>(), a);
+static void row(const TPArgs& a, int gy, Chain& q) {
+  q.launch(k_row<N, MODE>, dim3(N / Geo2<N>::RB, gy), NT2, row_smem_bytes<N>(), a);
 }
 template <int N, int MODE>
-static void col(const TPArgs& a, int gy, Seq& q) {
-  q.launch(k_col<N, MODE>, dim3(N / Geo2<N>::CW, gy), col_smem_bytes<N>(), a);
+static void col(const TPArgs& a, int gy, Chain& q) {
+  q.launch(k_col<N, MODE>, dim3(N / Geo2<N>::CW, gy), NT2, col_smem_bytes<N>(), a);
 }
 
 template <int N, class F>
@@ -1032,7 +998,7 @@ static bool encode_tile_map(CUtensorMap* m, const void* base, unsigned long long
 }
 
 template <int N>
-static cudaError_t twopass_t(TPArgs a, cudaStream_t s, cudaEvent_t ev0, cudaEvent_t ev1, cudaEvent_t meas_ready,
+static cudaError_t twopass_t(TPArgs a, Chain& q, cudaEvent_t ev0, cudaEvent_t ev1, cudaEvent_t meas_ready,
                              const cudaEvent_t* meas_part, int n_meas_part) {
   const bool far = a.farfield != 0;
   const int B = a.B, M = a.M, L = a.L;
@@ -1069,15 +1035,18 @@ static cudaError_t twopass_t(TPArgs a, cudaStream_t s, cudaEvent_t ev0, cudaEven
   // the detector passes (and the separate loss pass) are the first readers of the measured
   // intensities: wait for their copy there, not before the forward passes
   cudaError_t werr = cudaSuccess;
-  Seq q(s);
+  const cudaStream_t s = q.s;
   auto wait_meas = [&]() {
     if (!meas_ready) return;
     const cudaError_t e = cudaStreamWaitEvent(s, meas_ready, 0);
     if (e != cudaSuccess && werr == cudaSuccess) werr = e;
     meas_ready = nullptr;
-    q.chained = false;
+    q.breaks();
   };
-  if (ev0) cudaEventRecord(ev0, s);
+  if (ev0) {
+    cudaEventRecord(ev0, s);
+    q.breaks();
+  }
   if (far) {
     row<N, R_PHAT>(a, M, q);
     col<N, C_PHAT>(a, M, q);
@@ -1111,7 +1080,7 @@ static cudaError_t twopass_t(TPArgs a, cudaStream_t s, cudaEvent_t ev0, cudaEven
           if (parts) {   // this distance's intensities only; the later ones are still arriving
             const cudaError_t e = cudaStreamWaitEvent(s, meas_part[d], 0);
             if (e != cudaSuccess && werr == cudaSuccess) werr = e;
-            q.chained = false;
+            q.breaks();
           }
           if (fuse && a.loss == 1) row<N, R_NEAR_DSEED_P>(a, B, q);
           else if (fuse) row<N, R_NEAR_DSEED>(a, B, q);
@@ -1122,8 +1091,7 @@ static cudaError_t twopass_t(TPArgs a, cudaStream_t s, cudaEvent_t ev0, cudaEven
   }
   wait_meas();   // (no-op when a detector pass already waited)
   if (!fuse) {
-    (k_loss2<<<dim3((unsigned)(NN / LOSS_PX), B * a.nd), 256, 0, s>>>(a), note_launch());
-    q.chained = false;
+    q.launch(k_loss2, dim3((unsigned)(NN / LOSS_PX), B * a.nd), 256, 0, a);
   }
   if (a.adj) {
     // ---------------- adjoint
@@ -1177,21 +1145,23 @@ static cudaError_t twopass_t(TPArgs a, cudaStream_t s, cudaEvent_t ev0, cudaEven
       }
     }
   }
-  if (ev1) cudaEventRecord(ev1, s);
-  q.chained = false;
+  if (ev1) {
+    cudaEventRecord(ev1, s);
+    q.breaks();
+  }
   if (a.adj) {
     const bool grads = a.posp && (a.gpos || a.gposd || a.gnf);
-    (k_final2<<<1 + (grads ? B * a.nd : 0), 128, 0, s>>>(a, nloss, ncol), note_launch());
-    if (want_gap && a.ggap) launch_gap_final(a.gapp, B, L - 1, ncol, a.ggap, s);
+    q.launch(k_final2, 1 + (grads ? B * a.nd : 0), 128, 0, a, nloss, ncol);
+    if (want_gap && a.ggap) launch_gap_final(a.gapp, B, L - 1, ncol, a.ggap, q);
     if (a.g_probe) {
       const size_t MNN = (size_t)M * NN;
       // per-element FP64 sum over the batch (deterministic), then back to real space
-      launch_qsum(a.qacc, a.qsum, B, MNN, s);
+      launch_qsum(a.qacc, a.qsum, B, MNN, q);
       if (far) {
         col<N, C_PG>(a, M, q);
         row<N, R_PG_OUT>(a, M, q);
       } else {
-        (k_add2<<<1024, 256, 0, s>>>(a.g_probe, a.qsum, MNN), note_launch());
+        q.launch(k_add2, 1024, 256, 0, a.g_probe, a.qsum, MNN);
       }
     }
   }
@@ -1199,7 +1169,7 @@ static cudaError_t twopass_t(TPArgs a, cudaStream_t s, cudaEvent_t ev0, cudaEven
   return e != cudaSuccess ? e : q.err != cudaSuccess ? q.err : werr;
 }
 
-cudaError_t launch_twopass(TPArgs a, cudaStream_t s, cudaEvent_t ev0, cudaEvent_t ev1, cudaEvent_t meas_ready,
+cudaError_t launch_twopass(TPArgs a, Chain& s, cudaEvent_t ev0, cudaEvent_t ev1, cudaEvent_t meas_ready,
                            const cudaEvent_t* meas_part, int n_meas_part) {
   switch (a.N) {
     case 256: return twopass_t<256>(a, s, ev0, ev1, meas_ready, meas_part, n_meas_part);

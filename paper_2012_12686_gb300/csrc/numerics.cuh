@@ -42,8 +42,8 @@ __device__ __forceinline__ float f64bits_to_f32(unsigned hi, unsigned lo) {
   if (e >= 255) r = (ah > 0x7FF00000u || (ah == 0x7FF00000u && lo != 0u)) ? 0x7FC00000u : 0x7F800000u;
   return __uint_as_float(sign | r);
 }
-__device__ __forceinline__ float f64_to_f32(const double* p) {   // load and narrow (read-only data)
-  const uint2 w = __ldg(reinterpret_cast<const uint2*>(p));
+__device__ __forceinline__ float f64_to_f32(const double* p) {   // load (from L2) and narrow
+  const uint2 w = __ldcg(reinterpret_cast<const uint2*>(p));
   return f64bits_to_f32(w.y, w.x);
 }
 
