@@ -263,6 +263,23 @@ __device__ __forceinline__ void path_body(const PathArgs& a) {
   const bool want_gap = GAP && adj && a.gapp != nullptr;
   float2* spck_b = want_gap ? a.spck + (size_t)b * M * ncp * NN : nullptr;
   float2* spsg_b = want_gap ? a.spseg + (size_t)b * M * cp * NN : nullptr;
+  // far field, one probe mode and measured data: the detector's frequency pass also forms the loss terms
+  // and the adjoint seed, so the detector field and dL/dI make no round trip through global memory (sparse
+  // slices at N = 128 510 -> 501 us; not in the pipelined form, whose sweep got slower, 1104 -> 1112 us)
+  const bool fuse = FAR && !PIPE && M == 1 && adj && a.I_meas != nullptr;
+  const float eps = a.eps, sc_loss = (float)a.inv_npix;
+  // per-pixel term of Eq. lsq_loss or Eq. poisson_loss, and dL/dI
+  auto loss_of = [&](float I, float im, float& dI) -> float {
+    if (a.loss == 0) {
+      const float sI = sqrtf(I + eps), sM = sqrtf(im + eps);
+      const float df = sI - sM;
+      dI = df / sI * sc_loss;
+      return df * df;
+    }
+    dI = (1.0f - im / (I + eps)) * sc_loss;
+    return I - im * logf(I + eps);
+  };
+  Kahan acc;
   if (rank == 0) {
   // ------------------------------------------------------------------ forward
   for (int m = 0; m < M; ++m) {
@@ -342,6 +359,27 @@ __device__ __forceinline__ void path_body(const PathArgs& a) {
         // Psi = (1/N) DFT_+[phi]; keep Psi, accumulate I over modes
         X::template fwd_pair<+1>(A, tw);
         X::row_sync();
+        if (fuse) {
+          const float* Im = a.I_meas + (size_t)b * NN;
+          float* Io = a.I_out ? a.I_out + (size_t)b * NN : nullptr;
+          const float sc = 2.0f * invN;
+          X::template r23<+1, -1>(A, tw, [&](V2& v, int ky, int t) {
+            const int p0 = ky * N + t;
+            float im[RX];
+#pragma unroll
+            for (int i = 0; i < RX; ++i) im[i] = __ldg(Im + p0 + KXS * i);
+#pragma unroll
+            for (int i = 0; i < RX; ++i) {
+              const float2 P = cscale(v[i], invN);
+              const float I = fmaf(P.x, P.x, P.y * P.y);
+              if (Io) Io[p0 + KXS * i] = I;
+              float dI;
+              acc.add(loss_of(I, im[i], dI));
+              v[i] = cscale(P, sc * dI);
+            }
+          });
+          break;
+        }
         float2* fm = a.far + ((size_t)b * M + m) * NN;
         X::template r23<+1, 0>(A, tw, [&](V2& v, int ky, int t) {
 #pragma unroll
@@ -402,10 +440,8 @@ __device__ __forceinline__ void path_body(const PathArgs& a) {
     const size_t npx = (size_t)nd * NN;
     const float* Im = a.I_meas ? a.I_meas + (size_t)b * npx : nullptr;
     float* Io = a.I_out ? a.I_out + (size_t)b * npx : nullptr;
-    const float eps = a.eps, sc = (float)a.inv_npix;
-    Kahan acc;
     constexpr int U = 4;   // pixels per thread whose loads are issued ahead of their stores
-    for (size_t p0 = threadIdx.x; p0 < npx; p0 += (size_t)U * NT) {
+    for (size_t p0 = threadIdx.x; p0 < npx && !fuse; p0 += (size_t)U * NT) {
       float Iv[U], mv[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
@@ -415,24 +451,13 @@ __device__ __forceinline__ void path_body(const PathArgs& a) {
       }
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-      const size_t p = p0 + (size_t)u * NT;
-      if (p >= npx) break;
-      const float I = Iv[u];
-      if (Io) Io[p] = I;
-      if (!Im) continue;
-      const float im = mv[u];
-      float term, dI;
-      if (a.loss == 0) {
-        const float sI = sqrtf(I + eps), sM = sqrtf(im + eps);
-        const float df = sI - sM;
-        term = df * df;
-        dI = df / sI;
-      } else {
-        term = I - im * logf(I + eps);
-        dI = 1.0f - im / (I + eps);
-      }
-      acc.add(term);
-      gI_b[p] = dI * sc;
+        const size_t p = p0 + (size_t)u * NT;
+        if (p >= npx) break;
+        if (Io) Io[p] = Iv[u];
+        if (!Im) continue;
+        float dI;
+        acc.add(loss_of(Iv[u], mv[u], dI));
+        gI_b[p] = dI;
       }
     }
     const double s = block_sum<NT>(acc.value(), red);
@@ -497,15 +522,17 @@ __device__ __forceinline__ void path_body(const PathArgs& a) {
     }
     if (FAR) {
       // phibar_{L-1} = (1/N) DFT_-[2 gI Psi]
-      const float2* fm = a.far + ((size_t)b * M + m) * NN;
-      const float sc = 2.0f * invN;
-      X::template r23<0, -1>(A, tw, [&](V2& v, int ky, int t) {
+      if (!fuse) {
+        const float2* fm = a.far + ((size_t)b * M + m) * NN;
+        const float sc = 2.0f * invN;
+        X::template r23<0, -1>(A, tw, [&](V2& v, int ky, int t) {
 #pragma unroll
-        for (int i = 0; i < RX; ++i) {
-          const int p = ky * N + t + KXS * i;
-          v[i] = cscale(fm[p], sc * gI_b[p]);
-        }
-      });
+          for (int i = 0; i < RX; ++i) {
+            const int p = ky * N + t + KXS * i;
+            v[i] = cscale(fm[p], sc * gI_b[p]);
+          }
+        });
+      }
       X::row_sync();
       X::template inv_pair<-1>(A, tw);
     } else {
