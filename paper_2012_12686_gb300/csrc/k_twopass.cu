@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(NT2, row_minb<N, MODE>()) k_row(const TPArgs a
     dst = a.FA + fo;
     so = (FAR && j == a.L - 1) ? +1 : -1;
   } else if (MODE == R_RC_FIRST) {
-    src = a.ckpt + (((size_t)b * a.M + m) * a.ncp + a.s) * NN;
+    src = (!FAR && j == 0) ? a.probe + (size_t)m * NN : a.ckpt + (((size_t)b * a.M + m) * a.ncp + a.s) * NN;
     in_freq = false;
     dst = a.FR + fo;
   } else if (MODE == R_RC) {
@@ -312,7 +312,9 @@ __global__ void __launch_bounds__(NT2, row_minb<N, MODE>()) k_row(const TPArgs a
     const size_t orow = ((size_t)gz * a.Ly + gy) * a.Lx + p0x + t;   // voxel of pixel k: orow + N2 k
     const float2* psrc = nullptr;
     if (ADJ)
-      psrc = (j == a.j0) ? a.ckpt + (((size_t)b * a.M + m) * a.ncp + a.s) * NN
+      psrc = (!FAR && j == 0) ? a.probe + (size_t)m * NN   // psi_0 is the illumination (no checkpoint: 1.6 % of a
+                                                        // one-slice call on 8 problems of 1024 x 1024)
+             : (j == a.j0) ? a.ckpt + (((size_t)b * a.M + m) * a.ncp + a.s) * NN
                          : a.seg + (((size_t)b * a.M + m) * a.cp + (j - a.j0)) * NN;
     float2 Tv[2][CH], pv[2][ADJ ? CH : 1];
     float gdv[2][ADJ ? CH : 1], gbv[2][ADJ ? CH : 1];
@@ -348,7 +350,7 @@ __global__ void __launch_bounds__(NT2, row_minb<N, MODE>()) k_row(const TPArgs a
     // spatial ops; x = N2 k + t
     if (MODULATES) {
       float2* keep = nullptr;   // psi_j: checkpoint, segment slot or nowhere
-      if (MODE == R_FWD && a.adj) {
+      if (MODE == R_FWD && a.adj && (FAR || j > 0)) {
         if (j % a.cp == 0) keep = a.ckpt + (((size_t)b * a.M + m) * a.ncp + j / a.cp) * NN;
         else if (j > (a.ncp - 1) * a.cp) keep = a.seg + (((size_t)b * a.M + m) * a.cp + (j - (a.ncp - 1) * a.cp)) * NN;
       } else if (MODE == R_RC) {
