@@ -104,13 +104,15 @@ struct Region {
   size_t n;   // Lz * h * w
 };
 
-// (clamped to the volume whatever the words hold: they index it)
+// (clamped to the volume whatever the words hold: they index it).  Plain loads: every warp of the grid reads
+// these four words, and past L1 (__ldcg) they all met at one L2 line, 14.9 -> 27 us for the transmission
+// pass of 512 x 512 x 32.
 __device__ __forceinline__ Region region(const int* box, int Lz, int Ly, int Lx) {
   Region r;
-  r.y0 = min(max(__ldcg(box), 0), Ly);
-  r.h = min(max(__ldcg(box + 1), r.y0), Ly) - r.y0;
-  r.x0 = min(max(__ldcg(box + 2), 0), Lx);
-  r.w = min(max(__ldcg(box + 3), r.x0), Lx) - r.x0;
+  r.y0 = min(max(box[0], 0), Ly);
+  r.h = min(max(box[1], r.y0), Ly) - r.y0;
+  r.x0 = min(max(box[2], 0), Lx);
+  r.w = min(max(box[3], r.x0), Lx) - r.x0;
   r.n = (size_t)Lz * r.h * r.w;
   return r;
 }
