@@ -31,24 +31,18 @@ __device__ __forceinline__ void store_v(float* __restrict__ p, const float (&o)[
   else *p = o[0];
 }
 
-// Value and gradient.  A CTA takes a tile of 32 V x 8 columns (x, y) and walks zc planes of it: a warp
-// is one row, a thread V consecutive voxels.  The planes z - 1, z, z + 1 of delta and beta stay in
-// registers, the x neighbours come from the lanes beside (the tile's ends from one load), the y
-// neighbours from L1 where the tile holds them: 10 loads a voxel group instead of 14 + 4, and a fifth of
-// the L2 reads of a flat walk over the rows (which moved 60 bytes a voxel from L2 and was bound by it).
-// 512 x 512 x 32, weights, value and gradient (l1_weights and regularize): 192 -> 136 us; 80 registers
-// (three CTAs per SM), at 106 (two) 148 us.
-// V = 4 when Lx % 4 == 0 and the arrays are 16-byte aligned, else V = 1; the per-voxel arithmetic and
-// its order are the same.
-#ifndef REGB
-#define REGB 3
-#endif
-template <int V, bool TV>
-__global__ void __launch_bounds__(256, REGB) k_regularize(const float* __restrict__ d, const float* __restrict__ b,
+// Value and gradient, any alignment and row length.  A CTA takes a tile of 32 x 8 columns (x, y) and walks zc
+// planes of it: a warp is one row.  The planes z - 1, z, z + 1 of delta and beta stay in registers, the x
+// neighbours come from the lanes beside (the tile's ends from one load), the y neighbours from L1 where
+// the tile holds them.  One CTA per row with every neighbour read took 98 us for 32 x 512 x 509 and 23.7
+// for 64 x 130 x 126, this 91 and 20.5.  (Written for V consecutive voxels per thread; used with one.)
+template <bool TV>
+__global__ void __launch_bounds__(256) k_regularize(const float* __restrict__ d, const float* __restrict__ b,
                                                     const float* __restrict__ wd, const float* __restrict__ wb,
                                                     int Lz, int Ly, int Lx, float ad, float ab, float gam,
                                                     float invNo, float* __restrict__ gd, float* __restrict__ gb,
                                                     double* __restrict__ part, int zc) {
+  constexpr int V = 1;
   __shared__ double red[8];
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -171,6 +165,116 @@ __global__ void __launch_bounds__(256, REGB) k_regularize(const float* __restric
   }
 }
 
+// The same with four consecutive voxels of a row per thread, over the flat volume (Lx % 4 == 0 and
+// 16-byte aligned arrays): 128-bit loads of delta, beta, the weights, the neighbour rows and
+// planes and the gradients, the x neighbours across the group from two scalar loads.  Same
+// per-voxel arithmetic and order as k_regularize, whose tiles with four voxels a thread were slower
+// (73.7 against 71.5 us for 32 x 512 x 512, 43.0 against 36.8 for 8 x 700 x 700).
+template <bool TV>
+__global__ void __launch_bounds__(256) k_regularize4(const float* __restrict__ d, const float* __restrict__ b,
+                                                     const float* __restrict__ wd, const float* __restrict__ wb,
+                                                     int Lz, int Ly, int Lx, float ad, float ab, float gam,
+                                                     float invNo, float* __restrict__ gd, float* __restrict__ gb,
+                                                     double* __restrict__ part) {
+  __shared__ double red[8];
+  const int Lx4 = Lx >> 2;
+  const size_t sy = Lx, sz = (size_t)Lx * Ly;
+  const size_t n4 = (size_t)Ly * Lz * Lx4;
+  const float4 one4 = make_float4(1.f, 1.f, 1.f, 1.f);
+  Kahan acc;
+  for (size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x; q < n4; q += (size_t)gridDim.x * blockDim.x) {
+    const int r = (int)(q / Lx4), x0 = 4 * (int)(q - (size_t)r * Lx4);
+    const int z = r / Ly, y = r - z * Ly;
+    const size_t i = (size_t)r * Lx + x0;
+    const float4 vd = *reinterpret_cast<const float4*>(d + i), vb = *reinterpret_cast<const float4*>(b + i);
+    const float4 w1 = wd ? *reinterpret_cast<const float4*>(wd + i) : one4;
+    const float4 w2 = wb ? *reinterpret_cast<const float4*>(wb + i) : one4;
+    const float cd[4] = {vd.x, vd.y, vd.z, vd.w}, cb[4] = {vb.x, vb.y, vb.z, vb.w};
+    const float cw1[4] = {w1.x, w1.y, w1.z, w1.w}, cw2[4] = {w2.x, w2.y, w2.z, w2.w};
+    float term[4], g1[4], g2[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      term[e] = ad * cw1[e] * fabsf(cd[e]) + ab * cw2[e] * fabsf(cb[e]);
+      g1[e] = ad * cw1[e] * sgn(cd[e]);
+      g2[e] = ab * cw2[e] * sgn(cb[e]);
+    }
+    if (TV) {
+      // x neighbours: within the group, and one scalar on each side
+      float nd[6], nb[6];   // nd[e + 1] = delta at x0 + e, e = -1..4
+      nd[0] = x0 > 0 ? d[i - 1] : 0.f;
+      nb[0] = x0 > 0 ? b[i - 1] : 0.f;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        nd[e + 1] = cd[e];
+        nb[e + 1] = cb[e];
+      }
+      nd[5] = x0 + 4 < Lx ? d[i + 4] : 0.f;
+      nb[5] = x0 + 4 < Lx ? b[i + 4] : 0.f;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int x = x0 + e;
+        if (x + 1 < Lx) {
+          const float fd = nd[e + 2] - cd[e], fb = nb[e + 2] - cb[e];
+          term[e] += gam * (fabsf(fd) + fabsf(fb));
+          g1[e] -= gam * sgn(fd);
+          g2[e] -= gam * sgn(fb);
+        }
+        if (x > 0) {
+          g1[e] += gam * sgn(cd[e] - nd[e]);
+          g2[e] += gam * sgn(cb[e] - nb[e]);
+        }
+      }
+      // y and z neighbours: whole groups of the adjacent rows and planes
+      const int pos[2] = {y, z}, lim[2] = {Ly, Lz};
+      const size_t st[2] = {sy, sz};
+#pragma unroll
+      for (int a = 0; a < 2; ++a) {
+        if (pos[a] + 1 < lim[a]) {
+          const float4 ud = *reinterpret_cast<const float4*>(d + i + st[a]);
+          const float4 ub = *reinterpret_cast<const float4*>(b + i + st[a]);
+          const float qd[4] = {ud.x, ud.y, ud.z, ud.w}, qb[4] = {ub.x, ub.y, ub.z, ub.w};
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const float fd = qd[e] - cd[e], fb = qb[e] - cb[e];
+            term[e] += gam * (fabsf(fd) + fabsf(fb));
+            g1[e] -= gam * sgn(fd);
+            g2[e] -= gam * sgn(fb);
+          }
+        }
+        if (pos[a] > 0) {
+          const float4 ud = *reinterpret_cast<const float4*>(d + i - st[a]);
+          const float4 ub = *reinterpret_cast<const float4*>(b + i - st[a]);
+          const float qd[4] = {ud.x, ud.y, ud.z, ud.w}, qb[4] = {ub.x, ub.y, ub.z, ub.w};
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            g1[e] += gam * sgn(cd[e] - qd[e]);
+            g2[e] += gam * sgn(cb[e] - qb[e]);
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) acc.add(term[e]);
+    if (gd) {
+      float4 od = *reinterpret_cast<float4*>(gd + i), ob = *reinterpret_cast<float4*>(gb + i);
+      od.x += g1[0] * invNo; od.y += g1[1] * invNo; od.z += g1[2] * invNo; od.w += g1[3] * invNo;
+      ob.x += g2[0] * invNo; ob.y += g2[1] * invNo; ob.z += g2[2] * invNo; ob.w += g2[3] * invNo;
+      *reinterpret_cast<float4*>(gd + i) = od;
+      *reinterpret_cast<float4*>(gb + i) = ob;
+    }
+  }
+  double v = acc.value();
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double s = 0.0;
+    for (int k = 0; k < 8; ++k) s += red[k];
+    part[blockIdx.x] = s;
+  }
+}
+
 // R = invNo * sum of the per-CTA partials: 256 threads, each adds a strided subset in order, then
 // a fixed shuffle tree and a fixed order over the warps (deterministic)
 __global__ void __launch_bounds__(256) k_reg_final(const double* __restrict__ part, int nparts, double invNo,
@@ -268,19 +372,30 @@ cudaError_t launch_regularize(const float* d, const float* b, const float* wd, c
   const size_t n = (size_t)Lz * Ly * Lx;
   const float invNo = (float)(1.0 / (double)n);
   const bool vec = Lx % 4 == 0 && aligned16(d) && aligned16(b) && aligned16(wd) && aligned16(wb) && aligned16(gd) && aligned16(gb);
-  const int V = vec ? 4 : 1;
+  auto final_sum = [&](unsigned grid) {
+    if (loss) (k_reg_final<<<1, 256, 0, s>>>(part, (int)grid, 1.0 / (double)n, loss), note_launch());
+    return cudaGetLastError();
+  };
+  if (vec) {
+    const unsigned grid = reg_grid(n);
+    if (gam != 0.0)
+      (k_regularize4<true><<<grid, 256, 0, s>>>(d, b, wd, wb, Lz, Ly, Lx, (float)ad, (float)ab, (float)gam, invNo, gd,
+                                                gb, part), note_launch());
+    else
+      (k_regularize4<false><<<grid, 256, 0, s>>>(d, b, wd, wb, Lz, Ly, Lx, (float)ad, (float)ab, 0.f, invNo, gd, gb,
+                                                 part), note_launch());
+    return final_sum(grid);
+  }
   // planes per tile: as many as leave the chip eight CTAs per SM (fewer planes re-read more of their neighbours)
-  const long long tiles = (long long)((Lx + 32 * V - 1) / (32 * V)) * ((Ly + 7) / 8);
+  const long long tiles = (long long)((Lx + 31) / 32) * ((Ly + 7) / 8);
   int zc = 16;
   while (zc > 2 && tiles * ((Lz + zc - 1) / zc) < 152 * 8) zc /= 2;
   const unsigned grid = (unsigned)std::min<long long>(tiles * ((Lz + zc - 1) / zc), reg_grid(n));
   auto run = [&](auto kernel, float g) {
     (kernel<<<grid, 256, 0, s>>>(d, b, wd, wb, Lz, Ly, Lx, (float)ad, (float)ab, g, invNo, gd, gb, part, zc), note_launch());
   };
-  if (gam != 0.0) vec ? run(k_regularize<4, true>, (float)gam) : run(k_regularize<1, true>, (float)gam);
-  else vec ? run(k_regularize<4, false>, 0.f) : run(k_regularize<1, false>, 0.f);
-  if (loss) (k_reg_final<<<1, 256, 0, s>>>(part, (int)grid, 1.0 / (double)n, loss), note_launch());
-  return cudaGetLastError();
+  gam != 0.0 ? run(k_regularize<true>, (float)gam) : run(k_regularize<false>, 0.f);
+  return final_sum(grid);
 }
 
 cudaError_t launch_l1_weights(const float* d, const float* b, size_t n, float eps, float* part, float* wd, float* wb,
