@@ -1,5 +1,5 @@
-"""Regularizer and l1-weight kernels at the edges of their tiles (32 V x 8 columns, V = 4 or 1 by Lx, a
-few planes), against the FP64 oracle.
+"""Regularizer and l1-weight kernels at the edges of their tiles (32 x 8 columns and a few planes; 128-bit
+groups where Lx % 4 == 0), against the FP64 oracle.
 
 Tolerances: a gradient value is a sum of at most seven FP32 terms scaled once, so 8 x 2^-24 < 1e-6
 of its size; the value is Kahan-compensated; a weight takes one addition and one division.
