@@ -178,6 +178,9 @@ struct Field {
 // ---------------------------------------------------------------------------
 // Passes.  Signs are compile-time: S = -1 (DFT_-), +1 (DFT_+), 0 (stage skipped).
 //
+// A pass with a barrier inside takes its shared-memory pointers without __restrict__: with it the compiler
+// may move a load across the barrier, above the other threads' writes that the barrier waits for.
+//
 // Column pass "14": tasks (x, t < N2); v[k] <-> sample y = N2*k + t.
 //   pre(pa, pb, x, t): issues the task's global loads, before the CTA barrier that opens the pass
 //   op(v, pa, pb, x, t): spatial pointwise op on natural samples
@@ -200,7 +203,7 @@ struct Tpt {
 };
 
 template <int N, int S4, int S1, bool LOAD, bool STORE, class Pre, class Op>
-__device__ __forceinline__ void pass_c14(float2* __restrict__ A, const float2* __restrict__ tw, Pre pre, Op op) {
+__device__ __forceinline__ void pass_c14(float2* A, const float2* tw, Pre pre, Op op) {
   using F = Field<N>;
   constexpr int N1 = F::N1, N2 = F::N2, LD = F::LD;
   using P = Tpt<N * N2, F::NT>;

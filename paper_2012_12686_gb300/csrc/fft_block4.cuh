@@ -66,7 +66,7 @@ __device__ __forceinline__ void stagger() {
 //   LOAD = false: the samples come from op (no shared read, no y-S4)
 //   S1 != 0: y-S1 and store; S1 == 0: store natural samples; STORE = false: no store
 template <int S4, int S1, bool LOAD, bool STORE, class Pre, class Op>
-__device__ __forceinline__ void pass4_a(float2* __restrict__ A, const float2* __restrict__ tw, Pre pre, Op op) {
+__device__ __forceinline__ void pass4_a(float2* A, const float2* tw, Pre pre, Op op) {
   using G = G128;
   constexpr int N = G::N, LD = G::LD, NY1 = G::NY1, NY2 = G::NY2, Q = (N * NY2) / G::NT;
   static_assert(Q == 2, "two tasks per thread");
@@ -291,8 +291,7 @@ __device__ __forceinline__ float2* row64_scratch() {
 }
 
 template <int S>
-__device__ __forceinline__ void row64_line(float2 (&v)[8], const float2 (&wt)[8], float2* __restrict__ ws, int g,
-                                           int a) {
+__device__ __forceinline__ void row64_line(float2 (&v)[8], const float2 (&wt)[8], float2* ws, int g, int a) {
   dft<8, S>(v);
 #pragma unroll
   for (int k = 1; k < 8; ++k) v[k] = S < 0 ? cmul(v[k], wt[k]) : cmulc(v[k], wt[k]);   // twiddle<S>
