@@ -306,6 +306,7 @@ int enqueue(const Plan& pl, const Object& obj, const Tables& tab, const CallPtrs
   int* status = c.status ? c.status : reinterpret_cast<int*>(W(pl.off_status));
   bool join_side = false;   // the call's stream waits for the side stream's last kernels
   Chain s(stream), s2(c.side ? c.side : stream);
+  s2.overlap = s.overlap;   // the side stream joins a capture of the call's stream only with the fork below
   float2* phat = reinterpret_cast<float2*>(W(pl.off_phat));
   // the probe transform needs only the probe: on the side stream it overlaps the passes below
     // (only beside box kernels that take longer than the forks and joins)
