@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(Geo<N>::NT) k_probe_hat(const float2* __restri
 }
 
 // ---------------------------------------------------------------------------- probe gradient
-// qsum[m][p] = sum_b qacc[b][m][p] in FP64, fixed order
+// qsum[m][p] = sum_b qacc[b][m][p], fixed order
 // Block of 256 threads = 32 consecutive elements x 8 batch chunks; each thread sums its chunk
 // Kahan-compensated in FP32 (loads issued four at a time), then the 8 partials of an element are
 // added in FP64 in chunk order (deterministic).
@@ -80,21 +80,50 @@ __global__ void __launch_bounds__(256) k_qsum(const float2* qacc, float2* __rest
   }
 }
 
-// The same for a batch too small to split: a thread per element, the batch in its own order.
+// Running complex sum held as s + e + f: what an addition to s rounds off goes to e, what that addition rounds
+// off to f, both exactly (Knuth's TwoSum), so a sum of n terms is off by at most n^3 2^-72 of their sizes (an
+// FP64 sum: n 2^-53), whatever their order and signs.  A Kahan sum drops the low part of the running sum
+// when the next term is larger, which an element whose terms cancel shows in full (4 to 13 % of the worst
+// among 10^6 sums of eight normal terms).
+__device__ __forceinline__ void two_sum(float2 a, float2 b, float2& s, float2& e) {   // s + e == a + b
+  s = cadd(a, b);
+  const float2 bb = csub(s, a);
+  e = cadd(csub(a, csub(s, bb)), csub(b, bb));
+}
+struct Sum3 {
+  float2 s, e = {0.f, 0.f}, f = {0.f, 0.f};
+  __device__ __forceinline__ explicit Sum3(float2 first) : s(first) {}
+  __device__ __forceinline__ void add(float2 x) {
+    float2 r, q;
+    two_sum(s, x, s, r);
+    two_sum(e, r, e, q);
+    f = cadd(f, q);
+  }
+  // the sum rounded once, within 2^-24 of an ulp: e (which exceeds s where s cancels) and f are moved up
+  // exactly until each part is below half an ulp of the one above
+  __device__ __forceinline__ float2 value() const {
+    float2 s1, e1, e2, f2, s2, e3;
+    two_sum(s, e, s1, e1);
+    two_sum(e1, f, e2, f2);
+    two_sum(s1, e2, s2, e3);
+    return cadd(s2, cadd(e3, f2));
+  }
+};
+
+// The same for a batch of at most eight, whose chunks would hold one value or none: a thread per element, the
+// batch in its own order, to the accuracy of the FP64 sum over chunks of one value (Sum3).  FP32 adds: a
+// call on 8 holograms of 1024 x 1024 at two distances takes 428 us, with the sum on the FP64 pipe 452, with
+// a Kahan sum 426.
 __global__ void __launch_bounds__(256) k_qsum_few(const float2* qacc, float2* __restrict__ qsum, int B,
                                                   size_t MNN) {
   allow_next();
   after_previous();
   const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
   if (i >= MNN) return;
-  Kahan sr, si;
+  Sum3 t(__ldcg(qacc + i));
 #pragma unroll 4
-  for (int b = 0; b < B; ++b) {
-    const float2 v = __ldcg(qacc + (size_t)b * MNN + i);
-    sr.add(v.x);
-    si.add(v.y);
-  }
-  qsum[i] = make_float2((float)sr.value(), (float)si.value());
+  for (int b = 1; b < B; ++b) t.add(__ldcg(qacc + (size_t)b * MNN + i));
+  qsum[i] = t.value();
 }
 
 // g_gap[j] = sum of gap j's partials over the positions and column CTAs, one CTA per gap, threads strided

@@ -1157,7 +1157,7 @@ static cudaError_t twopass_t(TPArgs a, Chain& q, cudaEvent_t ev0, cudaEvent_t ev
     if (want_gap && a.ggap) launch_gap_final(a.gapp, B, L - 1, ncol, a.ggap, q);
     if (a.g_probe) {
       const size_t MNN = (size_t)M * NN;
-      // per-element FP64 sum over the batch (deterministic), then back to real space
+      // per-element compensated sum over the batch (deterministic), then back to real space
       launch_qsum(a.qacc, a.qsum, B, MNN, q);
       if (far) {
         col<N, C_PG>(a, M, q);

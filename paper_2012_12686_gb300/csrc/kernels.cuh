@@ -249,7 +249,8 @@ cudaError_t launch_regularize(const float* d, const float* b, const float* wd, c
 // W = max|C| / (|C| + eps) for C = delta and beta; part needs 2 reg_parts(n) floats
 cudaError_t launch_l1_weights(const float* d, const float* b, size_t n, float eps, float* part, float* wd, float* wb,
                               cudaStream_t s);
-// qsum[i] = sum_b qacc[b][i] in FP64, fixed order
+// qsum[i] = sum_b qacc[b][i] in a fixed order: up to eight terms as an FP64 sum rounded once, more in eight
+// Kahan-compensated FP32 chunks that are added in FP64
 cudaError_t launch_qsum(const float2* qacc, float2* qsum, int B, size_t MNN, Chain& s);
 int path_smem_bytes(int N);
 // whole two-pass loss/gradient (adj = 1) or forward (adj = 0) sequence for N in {256, 512, 1024}
