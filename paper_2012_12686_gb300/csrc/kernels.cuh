@@ -5,6 +5,7 @@
 #include <atomic>
 #include <cstddef>
 #include <cstdint>
+#include <utility>
 
 namespace adorym {
 
@@ -51,7 +52,7 @@ struct Chain {
     at.val.programmaticStreamSerializationAllowed = 1;
     c.attrs = &at;
     c.numAttrs = overlap && chained ? 1 : 0;
-    const cudaError_t e = cudaLaunchKernelEx(&c, kernel, P(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&c, kernel, std::forward<A>(args)...);   // implicit conversions only
     if (e != cudaSuccess && err == cudaSuccess) err = e;
     note_launch();
     chained = true;
