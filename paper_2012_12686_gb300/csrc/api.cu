@@ -284,8 +284,14 @@ int get_tables(adorym_ctx* ctx, const adorym_problem& p, Tables* out) {
   return ADORYM_OK;
 }
 
-// Boxes from which the probe kernels run on the side stream.  Below, the box kernels are shorter than two
-// forks and joins, and the call is one chain.
+// Volumes from which the probe kernels run on the side stream, beside the box kernels.  (The volume stands for
+// the batch's box, which only the device knows.)  Below, the call is one chain: its forks and joins
+// are 4 to 14 us of a call that is waited for, while calls in a row gain from the overlap where the box
+// kernels are long enough.  Chain / side stream, us, one slice and lsq: N = 32, 64 x 64, 49 positions 30.7 /
+// 32.1 (waited for 45 / 52); 4 x 128 x 128 53 / 48 (62 / 67); 360 x 360 42 / 34 (48 / 52); 400 x 400 37 / 35
+// (48 / 52).  N = 64, 200 positions in 360 x 360 61 / 64 (75 / 83).  N = 128, where the one-CTA probe kernels take
+// 13 to 19 us, at most 3 % apart either way: 4 positions in 144 x 144 97.1 / 94.7, 49 in 300 x 300 99.9 / 100.0,
+// 64 in 2 x 250 x 250 124.7 / 126.3, 64 in 2 x 400 x 400 126.5 / 124.8 (waited for 139.5 / 141).
 constexpr size_t kSideVoxels = (size_t)1 << 17;
 
 int enqueue(const Plan& pl, const Object& obj, const Tables& tab, const CallPtrs& c, char* ws, cudaStream_t stream,
@@ -309,7 +315,6 @@ int enqueue(const Plan& pl, const Object& obj, const Tables& tab, const CallPtrs
   s2.overlap = s.overlap;   // the side stream joins a capture of the call's stream only with the fork below
   float2* phat = reinterpret_cast<float2*>(W(pl.off_phat));
   // the probe transform needs only the probe: on the side stream it overlaps the passes below
-    // (only beside box kernels that take longer than the forks and joins)
   const bool side = c.side && !two_pass(p.N) && V >= kSideVoxels;
   if (side && pl.far) {
     if ((rc = chk(cudaEventRecord(c.ev_side[0], stream), "fork"))) return rc;
