@@ -35,73 +35,70 @@ __device__ __forceinline__ void store_v(float* __restrict__ p, const float (&o)[
 // planes of it: a warp is one row.  The planes z - 1, z, z + 1 of delta and beta stay in registers, the x
 // neighbours come from the lanes beside (the tile's ends from one load), the y neighbours from L1 where
 // the tile holds them.  One CTA per row with every neighbour read took 98 us for 32 x 512 x 509 and 23.7
-// for 64 x 130 x 126, this 91 and 20.5.  (Written for V consecutive voxels per thread; used with one.)
+// for 64 x 130 x 126, this 91 and 20.5.
 template <bool TV>
 __global__ void __launch_bounds__(256) k_regularize(const float* __restrict__ d, const float* __restrict__ b,
                                                     const float* __restrict__ wd, const float* __restrict__ wb,
                                                     int Lz, int Ly, int Lx, float ad, float ab, float gam,
                                                     float invNo, float* __restrict__ gd, float* __restrict__ gb,
                                                     double* __restrict__ part, int zc) {
-  constexpr int V = 1;
   __shared__ double red[8];
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const size_t sy = Lx, sz = (size_t)Lx * Ly;
-  const int gx = (Lx + 32 * V - 1) / (32 * V), gy = (Ly + 7) / 8, gz = (Lz + zc - 1) / zc;
+  const int gx = (Lx + 31) / 32, gy = (Ly + 7) / 8, gz = (Lz + zc - 1) / zc;
   const long long items = (long long)gx * gy * gz;
   Kahan acc;
   for (long long item = blockIdx.x; item < items; item += gridDim.x) {
     const int ix = (int)(item % gx), iy = (int)((item / gx) % gy), iz = (int)(item / ((long long)gx * gy));
-    const int x0 = (ix * 32 + lane) * V, y = iy * 8 + ty, z0 = iz * zc, z1 = min(z0 + zc, Lz);
-    const bool in = x0 < Lx && y < Ly;
-    size_t i = in ? ((size_t)z0 * Ly + y) * Lx + x0 : 0;
-    float cd[V] = {}, cb[V] = {}, pd[V] = {}, pb[V] = {}, nd[V] = {}, nb[V] = {};
+    const int x = ix * 32 + lane, y = iy * 8 + ty, z0 = iz * zc, z1 = min(z0 + zc, Lz);
+    const bool in = x < Lx && y < Ly;
+    size_t i = in ? ((size_t)z0 * Ly + y) * Lx + x : 0;
+    float cd = 0.f, cb = 0.f, pd = 0.f, pb = 0.f, nd = 0.f, nb = 0.f;   // this plane, the one before, the next
     if (in) {
-      load_v<V>(cd, d + i);
-      load_v<V>(cb, b + i);
+      cd = d[i];
+      cb = b[i];
       if (TV && z0 > 0) {
-        load_v<V>(pd, d + i - sz);
-        load_v<V>(pb, b + i - sz);
+        pd = d[i - sz];
+        pb = b[i - sz];
       }
     }
     for (int z = z0; z < z1; ++z, i += sz) {
-      float w1[V], w2[V], od[V] = {}, ob[V] = {}, ud[V] = {}, ub[V] = {}, vd[V] = {}, vb[V] = {};
-      float ld = 0.f, lb = 0.f, rd = 0.f, rb = 0.f;   // x neighbours beyond the warp's row piece
-#pragma unroll
-      for (int e = 0; e < V; ++e) w1[e] = w2[e] = 1.f;
+      float w1 = 1.f, w2 = 1.f, od = 0.f, ob = 0.f, ud = 0.f, ub = 0.f, vd = 0.f, vb = 0.f;
+      float ld = 0.f, lb = 0.f, rd = 0.f, rb = 0.f;   // x neighbours
       if (in) {
         if (z + 1 < (TV ? Lz : z1)) {
-          load_v<V>(nd, d + i + sz);
-          load_v<V>(nb, b + i + sz);
+          nd = d[i + sz];
+          nb = b[i + sz];
         }
         if (TV) {
           if (y + 1 < Ly) {
-            load_v<V>(ud, d + i + sy);
-            load_v<V>(ub, b + i + sy);
+            ud = d[i + sy];
+            ub = b[i + sy];
           }
           if (y > 0) {
-            load_v<V>(vd, d + i - sy);
-            load_v<V>(vb, b + i - sy);
+            vd = d[i - sy];
+            vb = b[i - sy];
           }
-          if (lane == 0 && x0 > 0) {
+          if (lane == 0 && x > 0) {
             ld = d[i - 1];
             lb = b[i - 1];
           }
-          if (lane == 31 && x0 + V < Lx) {
-            rd = d[i + V];
-            rb = b[i + V];
+          if (lane == 31 && x + 1 < Lx) {
+            rd = d[i + 1];
+            rb = b[i + 1];
           }
         }
-        if (wd) load_v<V>(w1, wd + i);
-        if (wb) load_v<V>(w2, wb + i);
+        if (wd) w1 = wd[i];
+        if (wb) w2 = wb[i];
         if (gd) {
-          load_v<V>(od, gd + i);
-          load_v<V>(ob, gb + i);
+          od = gd[i];
+          ob = gb[i];
         }
       }
       if (TV) {
-        const float a = __shfl_up_sync(full, cd[V - 1], 1), c = __shfl_up_sync(full, cb[V - 1], 1);
-        const float f = __shfl_down_sync(full, cd[0], 1), g = __shfl_down_sync(full, cb[0], 1);
+        const float a = __shfl_up_sync(full, cd, 1), c = __shfl_up_sync(full, cb, 1);
+        const float f = __shfl_down_sync(full, cd, 1), g = __shfl_down_sync(full, cb, 1);
         if (lane > 0) {
           ld = a;
           lb = c;
@@ -112,45 +109,38 @@ __global__ void __launch_bounds__(256) k_regularize(const float* __restrict__ d,
         }
       }
       if (in) {
-#pragma unroll
-        for (int e = 0; e < V; ++e) {
-          const float qd = cd[e], qb = cb[e];
-          float term = ad * w1[e] * fabsf(qd) + ab * w2[e] * fabsf(qb);
-          float g1 = ad * w1[e] * sgn(qd), g2 = ab * w2[e] * sgn(qb);
-          if (TV) {
-            auto ahead = [&](float hd, float hb) {   // forward difference of this voxel
-              const float fd = hd - qd, fb = hb - qb;
-              term += gam * (fabsf(fd) + fabsf(fb));
-              g1 -= gam * sgn(fd);
-              g2 -= gam * sgn(fb);
-            };
-            auto behind = [&](float hd, float hb) {   // forward difference of the voxel before
-              g1 += gam * sgn(qd - hd);
-              g2 += gam * sgn(qb - hb);
-            };
-            if (x0 + e + 1 < Lx) ahead(e + 1 < V ? cd[(e + 1) % V] : rd, e + 1 < V ? cb[(e + 1) % V] : rb);
-            if (x0 + e > 0) behind(e > 0 ? cd[(e + V - 1) % V] : ld, e > 0 ? cb[(e + V - 1) % V] : lb);
-            if (y + 1 < Ly) ahead(ud[e], ub[e]);
-            if (y > 0) behind(vd[e], vb[e]);
-            if (z + 1 < Lz) ahead(nd[e], nb[e]);
-            if (z > 0) behind(pd[e], pb[e]);
-          }
-          acc.add(term);
-          od[e] += g1 * invNo;
-          ob[e] += g2 * invNo;
+        float term = ad * w1 * fabsf(cd) + ab * w2 * fabsf(cb);
+        float g1 = ad * w1 * sgn(cd), g2 = ab * w2 * sgn(cb);
+        if (TV) {
+          auto ahead = [&](float hd, float hb) {   // forward difference of this voxel
+            const float fd = hd - cd, fb = hb - cb;
+            term += gam * (fabsf(fd) + fabsf(fb));
+            g1 -= gam * sgn(fd);
+            g2 -= gam * sgn(fb);
+          };
+          auto behind = [&](float hd, float hb) {   // forward difference of the voxel before
+            g1 += gam * sgn(cd - hd);
+            g2 += gam * sgn(cb - hb);
+          };
+          if (x + 1 < Lx) ahead(rd, rb);
+          if (x > 0) behind(ld, lb);
+          if (y + 1 < Ly) ahead(ud, ub);
+          if (y > 0) behind(vd, vb);
+          if (z + 1 < Lz) ahead(nd, nb);
+          if (z > 0) behind(pd, pb);
         }
+        acc.add(term);
+        od += g1 * invNo;
+        ob += g2 * invNo;
         if (gd) {
-          store_v<V>(gd + i, od);
-          store_v<V>(gb + i, ob);
+          gd[i] = od;
+          gb[i] = ob;
         }
       }
-#pragma unroll
-      for (int e = 0; e < V; ++e) {
-        pd[e] = cd[e];
-        pb[e] = cb[e];
-        cd[e] = nd[e];
-        cb[e] = nb[e];
-      }
+      pd = cd;
+      pb = cb;
+      cd = nd;
+      cb = nb;
     }
   }
   double v = acc.value();
