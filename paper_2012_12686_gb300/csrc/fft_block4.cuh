@@ -26,7 +26,9 @@
 // multislice loss and gradient 1.306 -> 1.230 ms, 256-position forward 0.796 -> 0.723 ms.
 // Shared layout: column c of a row at c + 8 (c / 32), row pitch 153 float2.  The 16 lanes of a
 // half-warp access of C (rows g < 8, t and t + 1) then sit at 9 g + 8 t mod 16, one per 8-byte bank
-// pair; A and B read 32 consecutive columns of one group, conflict-free at any pitch.
+// pair; A and B read 32 consecutive columns of one group, conflict-free at any pitch.  Two tables are not
+// conflict-free: C's hy (frequencies w + 16 g of the eight rows, all on one bank pair) and B's tw[2 tx]
+// (two to a bank pair).  The whole kernel counts 5.4 M conflicts in 122 M shared-memory wavefronts.
 //
 // Twiddles W_N^m = exp(-2 pi i m / N) come from the FP64-built table; every stage's twiddle index
 // t k stays below N.  C reads its own (t, k) table two entries per 128-bit load.
