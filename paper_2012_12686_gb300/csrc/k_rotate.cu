@@ -149,7 +149,6 @@ __global__ void __launch_bounds__(256) k_transmission(const float* __restrict__ 
                                                       float2* __restrict__ T, int Lz, int Ly, int Lx, float kdz,
                                                       float c, float s, const int* box,
                                                       double* __restrict__ zero_a, double* __restrict__ zero_b) {
-  allow_next();
   after_previous();
   const Region R = region(box, Lz, Ly, Lx);
   BoxChunks K(R, Lz);
@@ -217,6 +216,11 @@ __global__ void __launch_bounds__(256) k_transmission(const float* __restrict__ 
       }
     }
   }
+  // Only here: this grid fills the chip, and CTAs started before it is done go, several together, to the few
+  // SMs that are free first.  The fused kernel's small CTAs (N <= 32) then shared SMs while others stood idle:
+  // calls in a row, N = 32, 20 positions of 16 slices 143 us, 49 in 360 x 360 42, 200 near-field problems 66;
+  // with the signal here 92, 33 and 50 (and up to 3 % less at N = 64 .. 256, where a CTA has an SM for itself).
+  allow_next();
 }
 
 // transpose of the rotation, step 1 (per call, independent of y): for each unrotated node (z, x)
