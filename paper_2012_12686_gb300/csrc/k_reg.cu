@@ -7,6 +7,8 @@
 // atomics), per-CTA FP64 partial sums are added in a fixed order.
 #include <algorithm>
 #include <cstdint>
+#include <type_traits>
+#include <utility>
 
 #include "numerics.cuh"
 #include "kernels.cuh"
@@ -31,29 +33,33 @@ __device__ __forceinline__ void store_v(float* __restrict__ p, const float (&o)[
   else *p = o[0];
 }
 
-// Value and gradient, any alignment and row length.  A CTA takes a tile of 32 x 8 columns (x, y) and walks zc
-// planes of it: a warp is one row.  The planes z - 1, z, z + 1 of delta and beta stay in registers, the x
+// Value and gradient, any alignment and row length.  z (stride sz) is the axis that is walked and y (stride sy) the
+// other one, whichever the volume calls them.  A CTA's eight warps are RY rows times 8 / RY stretches of zc planes: a
+// warp walks zc planes of 32 columns of a row.  The planes z - 1, z, z + 1 of delta and beta stay in registers, the x
 // neighbours come from the lanes beside (the tile's ends from one load), the y neighbours from L1 where
-// the tile holds them.  One CTA per row with every neighbour read took 98 us for 32 x 512 x 509 and 23.7
-// for 64 x 130 x 126, this 91 and 20.5.
-template <bool TV>
+// the tile holds them.  One CTA per row with every neighbour read took 98 us for 32 x 512 x 509 and 52
+// for 33 x 300 x 301, this 88 and 38; eight rows for every volume took 35 us for 2000 x 1 x 301 (of which one
+// row is there), one CTA per row 16.6, this 16.4.  Item indices in 32 bits: in 64 their divisions were 6 %
+// (297 -> 284 us for 31 x 1025 x 1023).
+template <bool TV, int RY>
 __global__ void __launch_bounds__(256) k_regularize(const float* __restrict__ d, const float* __restrict__ b,
                                                     const float* __restrict__ wd, const float* __restrict__ wb,
-                                                    int Lz, int Ly, int Lx, float ad, float ab, float gam,
-                                                    float invNo, float* __restrict__ gd, float* __restrict__ gb,
-                                                    double* __restrict__ part, int zc) {
+                                                    int Lz, int Ly, int Lx, size_t sz, size_t sy, float ad, float ab,
+                                                    float gam, float invNo, float* __restrict__ gd,
+                                                    float* __restrict__ gb, double* __restrict__ part, int zc) {
   __shared__ double red[8];
   const unsigned full = 0xffffffffu;
-  const int lane = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  const size_t sy = Lx, sz = (size_t)Lx * Ly;
-  const int gx = (Lx + 31) / 32, gy = (Ly + 7) / 8, gz = (Lz + zc - 1) / zc;
-  const long long items = (long long)gx * gy * gz;
+  const int lane = threadIdx.x & 31, ty = (threadIdx.x >> 5) % RY, tz = (threadIdx.x >> 5) / RY;
+  const int pz = 8 / RY * zc;   // planes of a tile
+  const unsigned gx = (Lx + 31) / 32, gy = (Ly + RY - 1) / RY, gz = (Lz + pz - 1) / pz;
+  const unsigned items = gx * gy * gz;   // (below 2^30 for any volume that fits the card: 128 voxels and more each)
   Kahan acc;
-  for (long long item = blockIdx.x; item < items; item += gridDim.x) {
-    const int ix = (int)(item % gx), iy = (int)((item / gx) % gy), iz = (int)(item / ((long long)gx * gy));
-    const int x = ix * 32 + lane, y = iy * 8 + ty, z0 = iz * zc, z1 = min(z0 + zc, Lz);
-    const bool in = x < Lx && y < Ly;
-    size_t i = in ? ((size_t)z0 * Ly + y) * Lx + x : 0;
+  for (unsigned item = blockIdx.x; item < items; item += gridDim.x) {
+    const unsigned row = item / gx;
+    const int ix = (int)(item - row * gx), iz = (int)(row / gy), iy = (int)(row - (unsigned)iz * gy);
+    const int x = ix * 32 + lane, y = iy * RY + ty, z0 = iz * pz + tz * zc, z1 = min(z0 + zc, Lz);
+    const bool in = x < Lx && y < Ly && z0 < Lz;
+    size_t i = in ? z0 * sz + y * sy + x : 0;
     float cd = 0.f, cb = 0.f, pd = 0.f, pb = 0.f, nd = 0.f, nb = 0.f;   // this plane, the one before, the next
     if (in) {
       cd = d[i];
@@ -376,15 +382,35 @@ cudaError_t launch_regularize(const float* d, const float* b, const float* wd, c
                                                  part), note_launch());
     return final_sum(grid);
   }
-  // planes per tile: as many as leave the chip eight CTAs per SM (fewer planes re-read more of their neighbours)
-  const long long tiles = (long long)((Lx + 31) / 32) * ((Ly + 7) / 8);
+  // One plane is walked along y (1 x 3000 x 3001: 120 us as a walk of one plane, 90 so; one CTA per row 98).
+  int Lw = Lz, Lr = Ly;
+  size_t sw = (size_t)Lx * Ly, sr = Lx;
+  if (Lz == 1) {
+    std::swap(Lw, Lr);
+    std::swap(sw, sr);
+  }
+  // Rows per tile: a divisor of a small row count, so that no warp is without a row (4096 x 2 x 255: 59 -> 29 us,
+  // 100 x 5 x 1001 17.4 -> 16.7).
+  int ry = 8;
+  while (Lr < 8 && Lr % ry) ry /= 2;
+  // planes per walk: as many as leave the chip eight CTAs per SM (fewer planes re-read more of their neighbours)
+  const long long tiles = (long long)((Lx + 31) / 32) * ((Lr + ry - 1) / ry);
+  auto items = [&](int zc) { return tiles * ((Lw + 8 / ry * zc - 1) / (8 / ry * zc)); };
   int zc = 16;
-  while (zc > 2 && tiles * ((Lz + zc - 1) / zc) < 152 * 8) zc /= 2;
-  const unsigned grid = (unsigned)std::min<long long>(tiles * ((Lz + zc - 1) / zc), reg_grid(n));
+  while (zc > 2 && items(zc) < 152 * 8) zc /= 2;
+  const unsigned grid = (unsigned)std::min<long long>(items(zc), reg_grid(n));
   auto run = [&](auto kernel, float g) {
-    (kernel<<<grid, 256, 0, s>>>(d, b, wd, wb, Lz, Ly, Lx, (float)ad, (float)ab, g, invNo, gd, gb, part, zc), note_launch());
+    (kernel<<<grid, 256, 0, s>>>(d, b, wd, wb, Lw, Lr, Lx, sw, sr, (float)ad, (float)ab, g, invNo, gd, gb, part, zc), note_launch());
   };
-  gam != 0.0 ? run(k_regularize<true>, (float)gam) : run(k_regularize<false>, 0.f);
+  auto rows = [&](auto r) {
+    gam != 0.0 ? run(k_regularize<true, decltype(r)::value>, (float)gam) : run(k_regularize<false, decltype(r)::value>, 0.f);
+  };
+  switch (ry) {
+    case 8: rows(std::integral_constant<int, 8>()); break;
+    case 4: rows(std::integral_constant<int, 4>()); break;
+    case 2: rows(std::integral_constant<int, 2>()); break;
+    default: rows(std::integral_constant<int, 1>());
+  }
   return final_sum(grid);
 }
 
