@@ -285,13 +285,12 @@ int get_tables(adorym_ctx* ctx, const adorym_problem& p, Tables* out) {
 }
 
 // Volumes from which the probe kernels run on the side stream, beside the box kernels.  (The volume stands for
-// the batch's box, which only the device knows.)  Below, the call is one chain: its forks and joins
-// are 4 to 14 us of a call that is waited for, while calls in a row gain from the overlap where the box
-// kernels are long enough.  Chain / side stream, us, one slice and lsq: N = 32, 64 x 64, 49 positions 30.7 /
-// 32.1 (waited for 45 / 52); 4 x 128 x 128 53 / 48 (62 / 67); 360 x 360 42 / 34 (48 / 52); 400 x 400 37 / 35
-// (48 / 52).  N = 64, 200 positions in 360 x 360 61 / 64 (75 / 83).  N = 128, where the one-CTA probe kernels take
-// 13 to 19 us, at most 3 % apart either way: 4 positions in 144 x 144 97.1 / 94.7, 49 in 300 x 300 99.9 / 100.0,
-// 64 in 2 x 250 x 250 124.7 / 126.3, 64 in 2 x 400 x 400 126.5 / 124.8 (waited for 139.5 / 141).
+// the batch's box, which only the device knows.)  Below, the call is one chain: forks and joins are 2 to 8 us of
+// a call that is waited for and 0 to 3 of calls in a row.  Chain / side stream, us, calls in a row (waited for), lsq:
+// N = 32, 49 positions in 64 x 64 30.3 / 31.8 (44 / 51), in 4 x 128 x 128 47.5 / 48.6 (61 / 67), in 400 x 400 34.0 /
+// 34.5 (47 / 52); N = 64, 200 in 360 x 360 61 / 64 (75 / 82); N = 128, where the one-CTA probe kernels take 13 to
+// 19 us, 4 in 144 x 144 95 / 95 (109 / 111), 64 in 2 x 250 x 250 122.6 / 126 (137 / 138.5), 64 in 2 x 400 x 400
+// 126.6 / 124.9 (139.8 / 140.8): from there on, with longer box kernels, the overlap pays.
 constexpr size_t kSideVoxels = (size_t)1 << 17;
 
 int enqueue(const Plan& pl, const Object& obj, const Tables& tab, const CallPtrs& c, char* ws, cudaStream_t stream,
@@ -336,8 +335,10 @@ int enqueue(const Plan& pl, const Object& obj, const Tables& tab, const CallPtrs
     gd = acc;
     gb = acc + V;
   }
+  // (two-pass near field: the row kernel of all problems comes next; else a probe transform or the fused kernel)
+  const bool next_fills = two_pass(p.N) && !pl.far && (long long)p.B * twopass_columns(p.N) >= 2 * device_sms();
   if ((rc = chk(launch_transmission(obj.d, obj.b, T, p.Lz, p.Ly, p.Lx, (float)p.kdz, pl.tomo ? 1 : 0, (float)cth,
-                                    (float)sth, box, gd, gb, s),
+                                    (float)sth, box, gd, gb, next_fills, s),
                 "transmission")))
     return rc;
   // the fused kernel reads the measured intensities: wait for their copy before it (the pre-kernels

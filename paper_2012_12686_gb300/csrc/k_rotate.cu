@@ -148,7 +148,9 @@ template <bool ROT>
 __global__ void __launch_bounds__(256) k_transmission(const float* __restrict__ vd, const float* __restrict__ vb,
                                                       float2* __restrict__ T, int Lz, int Ly, int Lx, float kdz,
                                                       float c, float s, const int* box,
-                                                      double* __restrict__ zero_a, double* __restrict__ zero_b) {
+                                                      double* __restrict__ zero_a, double* __restrict__ zero_b,
+                                                      int next_fills) {
+  if (next_fills) allow_next();
   after_previous();
   const Region R = region(box, Lz, Ly, Lx);
   BoxChunks K(R, Lz);
@@ -216,11 +218,13 @@ __global__ void __launch_bounds__(256) k_transmission(const float* __restrict__ 
       }
     }
   }
-  // Only here: this grid fills the chip, and CTAs started before it is done go, several together, to the few
-  // SMs that are free first.  The fused kernel's small CTAs (N <= 32) then shared SMs while others stood idle:
-  // calls in a row, N = 32, 20 positions of 16 slices 143 us, 49 in 360 x 360 42, 200 near-field problems 66;
-  // with the signal here 92, 33 and 50 (and up to 3 % less at N = 64 .. 256, where a CTA has an SM for itself).
-  allow_next();
+  // Only here, unless the next kernel fills the chip as well: this grid does, and CTAs started before it is done
+  // go, several together, to the few SMs that are free first.  The fused kernel's small CTAs (N <= 32) then
+  // shared SMs while others stood idle: calls in a row, N = 32, 20 positions of 16 slices 143 us, 49 in 360 x 360
+  // 42, 200 near-field problems 66; with the signal here 92, 33 and 50, two problems of 512 x 512 at three
+  // distances 242 -> 230, and N = 64 .. 256 up to 3 % less.  8 problems of 1024 x 1024 (1024 row CTAs) lose their
+  // early start with it, 721 -> 724.
+  if (!next_fills) allow_next();
 }
 
 // transpose of the rotation, step 1 (per call, independent of y): for each unrotated node (z, x)
@@ -349,10 +353,10 @@ cudaError_t launch_bbox(const float* pos, int B, int N, int Ly, int Lx, int far,
 
 cudaError_t launch_transmission(const float* vd, const float* vb, float2* T, int Lz, int Ly, int Lx, float kdz,
                                 int rotate, float c, float sn, const int* box, double* zero_a, double* zero_b,
-                                Chain& s) {
+                                bool next_fills, Chain& s) {
   const unsigned grid = box_grid(Lz, Ly, Lx);
   return s.launch(rotate ? k_transmission<true> : k_transmission<false>, grid, 256, 0, vd, vb, T, Lz, Ly, Lx, kdz, c, sn,
-                  box, zero_a, zero_b);
+                  box, zero_a, zero_b, next_fills ? 1 : 0);
 }
 
 cudaError_t launch_rotate_adj(const double* gdr, const double* gbr, float* gd, float* gb, int Lz, int Ly, int Lx,

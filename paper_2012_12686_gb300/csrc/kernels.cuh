@@ -224,10 +224,11 @@ cudaError_t launch_bbox(const float* pos, int B, int N, int Ly, int Lx, int far,
                         int npos_values, int* status, bool clear, Chain& s, int* zero = nullptr, int nzero = 0);
 // T = exp(-kdz beta) exp(i kdz delta) over the box (Eq. ri_modulation), optionally after the
 // bilinear rotation of Eq. rotation_transform (rotate = 1); zero_a / zero_b (FP64 object-gradient
-// accumulators over the same box) are zeroed in the same pass when non-null
+// accumulators over the same box) are zeroed in the same pass when non-null; next_fills: the kernel launched
+// next has at least two CTAs per SM
 cudaError_t launch_transmission(const float* vd, const float* vb, float2* T, int Lz, int Ly, int Lx, float kdz,
                                 int rotate, float c, float sn, const int* box, double* zero_a, double* zero_b,
-                                Chain& s);
+                                bool next_fills, Chain& s);
 // The rotation's transpose per unrotated node (z, x), independent of y: the rotated-frame nodes
 // (z_t, x_t) that contribute and their bilinear weights.  The candidates lie in a 3 x 3 window
 // (|cos| + |sin| <= sqrt 2 on each side), so nine entries always suffice (up to five contribute
@@ -263,7 +264,7 @@ cudaError_t launch_twopass(TPArgs a, Chain& s, cudaEvent_t ev_start, cudaEvent_t
                            cudaEvent_t meas_ready = nullptr, const cudaEvent_t* meas_part = nullptr,
                            int n_meas_part = 0);
 cudaError_t prepare_twopass(int N);
-int twopass_columns(int N);   // column CTAs per field: partials per position of the column passes
+int twopass_columns(int N);   // column CTAs (and row CTAs) per field: partials per position of the column passes
 // set the dynamic shared-memory attributes of every kernel used for tile size N (call outside capture)
 cudaError_t prepare_path(int N, int farfield);
 
