@@ -336,7 +336,7 @@ int enqueue(const Plan& pl, const Object& obj, const Tables& tab, const CallPtrs
     gb = acc + V;
   }
   // (two-pass near field: the row kernel of all problems comes next; else a probe transform or the fused kernel)
-  const bool next_fills = two_pass(p.N) && !pl.far && (long long)p.B * twopass_columns(p.N) >= 2 * device_sms();
+  const bool next_fills = two_pass(p.N) && !pl.far && (long long)p.B * twopass_columns(p.N) >= device_sms();
   if ((rc = chk(launch_transmission(obj.d, obj.b, T, p.Lz, p.Ly, p.Lx, (float)p.kdz, pl.tomo ? 1 : 0, (float)cth,
                                     (float)sth, box, gd, gb, next_fills, s),
                 "transmission")))

@@ -222,8 +222,9 @@ __global__ void __launch_bounds__(256) k_transmission(const float* __restrict__ 
   // go, several together, to the few SMs that are free first.  The fused kernel's small CTAs (N <= 32) then
   // shared SMs while others stood idle: calls in a row, N = 32, 20 positions of 16 slices 143 us, 49 in 360 x 360
   // 42, 200 near-field problems 66; with the signal here 92, 33 and 50, two problems of 512 x 512 at three
-  // distances 242 -> 230, and N = 64 .. 256 up to 3 % less.  8 problems of 1024 x 1024 (1024 row CTAs) lose their
-  // early start with it, 721 -> 724.
+  // distances 242 -> 230, and N = 64 .. 256 up to 3 % less.  Row kernels of at least a CTA per SM lose their early
+  // start with it: 8 problems of 1024 x 1024 (1024 CTAs) 721 -> 724, 2 (256) 301 -> 309, 9 of 512 x 512 (288) 155.5 ->
+  // 159; 3 of 512 x 512 (96) gain, 255 -> 250.5.
   if (!next_fills) allow_next();
 }
 

@@ -225,7 +225,7 @@ cudaError_t launch_bbox(const float* pos, int B, int N, int Ly, int Lx, int far,
 // T = exp(-kdz beta) exp(i kdz delta) over the box (Eq. ri_modulation), optionally after the
 // bilinear rotation of Eq. rotation_transform (rotate = 1); zero_a / zero_b (FP64 object-gradient
 // accumulators over the same box) are zeroed in the same pass when non-null; next_fills: the kernel launched
-// next has at least two CTAs per SM
+// next has at least one CTA per SM
 cudaError_t launch_transmission(const float* vd, const float* vb, float2* T, int Lz, int Ly, int Lx, float kdz,
                                 int rotate, float c, float sn, const int* box, double* zero_a, double* zero_b,
                                 bool next_fills, Chain& s);
